@@ -8,7 +8,6 @@
 //   * the sums of eq. (7) for FP32 Gaussian samplers whose iteration starts
 //     from equal weights, one record per 256-particle warp tile (otherwise
 //     the quantisation pass forms them from the fixed-point weights),
-//   * the weighted covariance (diagnostic),
 //   * the iteration bookkeeping kernels (begin / commit, eq. (6) recycling).
 //
 // One thread owns one particle row at a time (grid-stride over N; the FP32
@@ -752,82 +751,6 @@ __global__ void __launch_bounds__(kFinBatchThreads) k_max_finalize_batch(const P
   max_finalize_body(a.part, nb[blockIdx.x], a.st);
 }
 
-// ---------------------------------------------------------------- covariance
-// cov_ab = sum_i w~_i (x_ia - mean_a)(x_ib - mean_b), w~_i = e^{log w_i - m} / s.
-// A block stages 128 rows at a time; each thread owns up to three (a <= b)
-// pairs and writes its block's sums to covpart[block][pair]; k_cov_finalize
-// adds the blocks in index order (no atomics: the result does not depend on
-// the order in which blocks run).
-__device__ __forceinline__ void cov_pair(int p, int d, int& pa, int& pb) {
-  int r = 0;
-  while (p >= d - r) {
-    p -= d - r;
-    ++r;
-  }
-  pa = r;
-  pb = r + p;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kPThreads) k_cov(ParticleArgs a, double* cov, double* __restrict__ covpart) {
-  constexpr int kChunk = 128;
-  if (!cov) cov = a.st->cov_out;
-  if (!cov || a.st->err) return;
-  __shared__ T rows[kChunk][kMaxD + 1];
-  __shared__ double wts[kChunk];
-  const int cur = a.st->cur;
-  const T* __restrict__ x = static_cast<const T*>(cur ? a.x[1] : a.x[0]);
-  const double m = a.st->m, s = a.st->est_s;
-  const int d = a.d;
-  const int npairs = d * (d + 1) / 2;
-  double acc[3] = {0.0, 0.0, 0.0};
-  int pa[3], pb[3];
-  for (int k = 0; k < 3; ++k) {
-    const int p = threadIdx.x + k * blockDim.x;
-    pa[k] = pb[k] = -1;
-    if (p < npairs) cov_pair(p, d, pa[k], pb[k]);
-  }
-  for (int64_t base = int64_t(blockIdx.x) * kChunk; base < a.n; base += int64_t(gridDim.x) * kChunk) {
-    if (threadIdx.x < kChunk) {
-      const int64_t i = base + threadIdx.x;
-      if (i < a.n) {
-        for (int c = 0; c < d; ++c) rows[threadIdx.x][c] = T(double(x[i * d + c]) - a.st->mean[c]);
-        const double lw = a.logw[i];
-        wts[threadIdx.x] = (lw == -INFINITY) ? 0.0 : exp(lw - m) / s;
-      } else {
-        wts[threadIdx.x] = 0.0;
-        for (int c = 0; c < d; ++c) rows[threadIdx.x][c] = T(0);
-      }
-    }
-    __syncthreads();
-    for (int k = 0; k < 3; ++k) {
-      if (pa[k] < 0) continue;
-      double v = 0.0;
-      for (int r = 0; r < kChunk; ++r) v += wts[r] * double(rows[r][pa[k]]) * double(rows[r][pb[k]]);
-      acc[k] += v;
-    }
-    __syncthreads();
-  }
-  for (int k = 0; k < 3; ++k)
-    if (pa[k] >= 0) covpart[size_t(blockIdx.x) * npairs + threadIdx.x + k * blockDim.x] = acc[k];
-}
-
-// Sums the per-block covariance partials in block order; fills both triangles.
-__global__ void k_cov_finalize(const DevState* st, double* cov, const double* __restrict__ covpart, int nblocks,
-                               int d) {
-  if (!cov) cov = st->cov_out;
-  if (!cov || st->err) return;
-  const int npairs = d * (d + 1) / 2;
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= npairs) return;
-  double v = 0.0;
-  for (int b = 0; b < nblocks; ++b) v += covpart[size_t(b) * npairs + p];
-  int pa, pb;
-  cov_pair(p, d, pa, pb);
-  cov[pa * d + pb] = v;
-  cov[pb * d + pa] = v;
-}
-
 // ---------------------------------------------------------------- bookkeeping
 __global__ void k_begin(DevState* st) {
   if (threadIdx.x == 0) st->t += 1;
@@ -989,18 +912,6 @@ cudaError_t launch_logistic_setup(TargetDev* tg, const float* X, const float* y,
 
 cudaError_t launch_max_finalize(const double* part, int nb, DevState* st, cudaStream_t s) {
   k_max_finalize<<<1, kFinThreads, 0, s>>>(part, nb, st);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cov(const ParticleArgs& a, double* cov, double* covpart, int grid, cudaStream_t s) {
-  if (a.dtype == SMC_F64)
-    k_cov<double><<<grid, kPThreads, 0, s>>>(a, cov, covpart);
-  else
-    k_cov<float><<<grid, kPThreads, 0, s>>>(a, cov, covpart);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const int npairs = a.d * (a.d + 1) / 2;
-  k_cov_finalize<<<(npairs + 127) / 128, 128, 0, s>>>(a.st, cov, covpart, grid, a.d);
   return cudaGetLastError();
 }
 

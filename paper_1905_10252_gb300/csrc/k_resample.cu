@@ -74,6 +74,25 @@ cudaError_t upload_expfx_table() {
   return e;
 }
 
+// The device copy of the table on the current device, for the kernels of
+// other translation units.
+cudaError_t expfx_table(const uint64_t** out) {
+  static const uint64_t* at[64] = {nullptr};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 0 && dev < 64 && at[dev]) {
+    *out = at[dev];
+    return cudaSuccess;
+  }
+  void* p = nullptr;
+  e = cudaGetSymbolAddress(&p, c_T);
+  if (e != cudaSuccess) return e;
+  *out = static_cast<const uint64_t*>(p);
+  if (dev >= 0 && dev < 64) at[dev] = *out;
+  return cudaSuccess;
+}
+
 __device__ __forceinline__ void load_table(uint64_t* T) {
   if (threadIdx.x < 128) T[threadIdx.x] = c_T[threadIdx.x];
   __syncthreads();

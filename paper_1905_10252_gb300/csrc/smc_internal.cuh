@@ -261,6 +261,24 @@ __device__ __forceinline__ void normals_f32(uint64_t seed, uint64_t t, uint32_t 
 }
 
 // ---------------------------------------------------------------- fixed-point exp
+// ~2^62 2^(-f 2^-64) for the 64 fraction bits f.
+__device__ __forceinline__ uint64_t exp2_neg_frac(uint64_t f, const uint64_t* __restrict__ T) {
+  const uint64_t LN2 = 0xB17217F7D1CF79ACull;  // round(ln(2) 2^64)
+  const unsigned j1 = unsigned(f >> 58);
+  const unsigned j2 = unsigned((f >> 52) & 63);
+  const uint64_t g = f & ((1ull << 52) - 1);
+  const uint64_t H = __umul64hi(g << 12, LN2);
+  constexpr uint64_t ONE = 1ull << 63;
+  uint64_t P = ONE / 24;
+  P = ONE / 6 - (__umul64hi(H, P) >> 12);
+  P = ONE / 2 - (__umul64hi(H, P) >> 12);
+  P = ONE - (__umul64hi(H, P) >> 12);
+  P = ONE - (__umul64hi(H, P) >> 12);
+  const uint64_t t1 = T[j1], t2 = T[64 + j2];
+  const uint64_t Tm = (__umul64hi(t1, t2) << 1) | ((t1 * t2) >> 63);
+  return __umul64hi(Tm, P);
+}
+
 // E(y) ~= 2^62 exp(y) for y <= 0, an integer in [0, 2^62]:
 //   a = -y; A = floor(a 2^57) from the bits of a; Z = A round(log2(e) 2^62)
 //   (z = a log2 e = Z 2^-119); k = integer part, f = 64 fraction bits;
@@ -284,23 +302,10 @@ __device__ __forceinline__ uint64_t expfx_a(double a, const uint64_t* __restrict
     A = sh >= 0 ? (mant << sh) : (sh > -64 ? (mant >> (-sh)) : 0);
   }
   const uint64_t L2E = 0x5C551D94AE0BF85Eull;  // round(log2(e) 2^62)
-  const uint64_t LN2 = 0xB17217F7D1CF79ACull;  // round(ln(2) 2^64)
   const uint64_t zlo = A * L2E, zhi = __umul64hi(A, L2E);
   const unsigned k = unsigned(zhi >> 55);
   const uint64_t f = (zhi << 9) | (zlo >> 55);
-  const unsigned j1 = unsigned(f >> 58);
-  const unsigned j2 = unsigned((f >> 52) & 63);
-  const uint64_t g = f & ((1ull << 52) - 1);
-  const uint64_t H = __umul64hi(g << 12, LN2);
-  constexpr uint64_t ONE = 1ull << 63;
-  uint64_t P = ONE / 24;
-  P = ONE / 6 - (__umul64hi(H, P) >> 12);
-  P = ONE / 2 - (__umul64hi(H, P) >> 12);
-  P = ONE - (__umul64hi(H, P) >> 12);
-  P = ONE - (__umul64hi(H, P) >> 12);
-  const uint64_t t1 = T[j1], t2 = T[64 + j2];
-  const uint64_t Tm = (__umul64hi(t1, t2) << 1) | ((t1 * t2) >> 63);
-  return __umul64hi(Tm, P) >> k;
+  return exp2_neg_frac(f, T) >> k;
 }
 
 __device__ __forceinline__ uint64_t expfx(double y, const uint64_t* __restrict__ T) {

@@ -196,7 +196,7 @@ cudaError_t launch_target_setup(TargetDev* tg, int kind, double nu, const double
 cudaError_t launch_logistic_setup(TargetDev* tg, const float* X, const float* y, int m, int d, double prior_var,
                                   float* Xw, float* yw, uint16_t* ximg, cudaStream_t s);
 cudaError_t launch_max_finalize(const double* part, int nb, DevState* st, cudaStream_t s);
-// eq. (7) covariance: grid blocks write covpart[grid][D(D+1)/2], then a fixed-order sum
+// eq. (7) covariance (k_moments.cu): grid blocks write covpart[grid][D(D+1)/2], then a fixed-order sum
 cudaError_t launch_cov(const ParticleArgs& a, double* cov, double* covpart, int grid, cudaStream_t s);
 cudaError_t launch_begin(DevState* st, cudaStream_t s);
 cudaError_t launch_commit(DevState* st, int d, int force_flip, int recycle, cudaStream_t s, int defer = 0);
@@ -236,6 +236,7 @@ cudaError_t launch_take_errors_batch(const ParticleArgs* pa, int32_t* errs, int 
 
 // k_resample.cu
 cudaError_t upload_expfx_table();  // once per device, outside stream capture
+cudaError_t expfx_table(const uint64_t** out);  // its device address (after the upload)
 cudaError_t launch_max_logw(const double* logw, int64_t n, double* part, int nb, DevState* st, cudaStream_t s);
 cudaError_t launch_quant_reduce(const QuantArgs& a, cudaStream_t s);
 cudaError_t launch_quant_finalize(const QuantArgs& a, int set_lse_prev, cudaStream_t s);
