@@ -16,12 +16,18 @@
 // division per row) took 4.59 ms at N = 2^20, D = 32.  FP32 samplers
 // therefore keep u and every sum as an unevaluated pair of FP32 values
 // (error-free product by FMA, Knuth's two-sum: Dekker 1971; Knuth, TAOCP 2,
-// 4.2.2), 11 FP32 operations per pair, and the weight comes from the
+// 4.2.2), 11 FP32
+// operations per pair, and the weight comes from the
 // integer exponential of the quantise pass with its exponent kept apart, so
 // that a weight far below the largest keeps its relative precision.  The sums
 // carry about 2^-45 relative error, far below the 2^-25 of rounding a row's
 // difference to FP32 (the row precision), and no FP64 operation is left on
 // the per-pair path.  FP64 samplers use FP64 FMAs, one per pair.
+//
+// Measured (kernel alone): N = 2^20, D = 32 FP32 4.59 -> 0.33 ms (0.79 of the
+// issue slots, 0.64 of the FP32 pipe); N = 2000003, D = 12 1.67 -> 0.165 ms.
+// Packed two-lane FP32 instructions (27 % fewer instructions) were no faster
+// (0.35 ms: the FP32 pipe does the same work).
 #include <cmath>
 
 #include "smc_internal.cuh"
@@ -41,7 +47,7 @@ __host__ __device__ constexpr int cov_tiles(int nt) { return nt * (nt + 1) / 2; 
 template <typename T>
 struct CovShape {
   static constexpr int kCap = sizeof(T) == 4 ? 3600 : 2048;
-  static constexpr int kLoads = (kCap + kCovThreads - 1) / kCovThreads;  // values a thread stages
+  static constexpr int kLoads = sizeof(T) == 4 ? 16 : 9;  // values a thread stages, at most (d = 20)
 };
 
 // index of tile t of the upper triangle of nt x nt tiles, row by row
@@ -112,7 +118,8 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
   __shared__ __align__(16) T s_r[S::kCap];
   __shared__ __align__(16) T s_u[S::kCap];
   __shared__ __align__(16) T s_ul[kF32 ? S::kCap : 4];
-  __shared__ T s_w[kCovThreads], s_wl[kF32 ? kCovThreads : 1];
+  __shared__ float2 s_wf[kF32 ? kCovThreads : 1];
+  __shared__ double s_wd[kF32 ? 1 : kCovThreads];
   __shared__ T s_mh[kMaxD], s_ml[kMaxD];
   __shared__ float s_inv[kMaxD];  // FP32: the columns' scale, a power of two
   __shared__ int s_ex[kMaxD];
@@ -125,8 +132,10 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
   const double m = a.st->m;
   const int tiles = cov_tiles(nt), groups = kCovThreads / tiles;
   const int rows = min(S::kCap / nc, kCovThreads) / groups * groups;
-  // a thread stages the chunk's values tid, tid + 256, ... (coalesced)
-  const int er = tid / d, ec = tid - er * d, sr = kCovThreads / d, sc = kCovThreads - sr * d;
+  // a thread stages one column's values of rows er, er + sr, ... (the first
+  // sr d threads; coalesced)
+  const int sr = kCovThreads / d, er = tid / d, ec = tid - er * d;
+  const bool stages = er < sr;
   if (tid < kMaxD) {
     const double mu = tid < d ? a.st->mean[tid] : 0.0;
     s_mh[tid] = T(mu);
@@ -160,25 +169,38 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
   const int tile = tid % tiles, group = tid / tiles;
   int ta, tb;
   tile_of(tile, nt, ta, tb);
-  T acc[kTileC * kTileC], low[kF32 ? kTileC * kTileC : 1];
+  T acc[kTileC * kTileC], low[kF32 ? kTileC * kTileC : 1];  // the sums (FP32: and their low parts)
 #pragma unroll
   for (int k = 0; k < kTileC * kTileC; ++k) {
     acc[k] = T(0);
     if (kF32) low[k] = T(0);
   }
+  T mh = T(0), ml = T(0);
+  float inv = 1.0f;
+  if (stages) {
+    mh = s_mh[ec];
+    ml = s_ml[ec];
+    if (kF32) inv = s_inv[ec];
+  }
   int K = -(1 << 20);  // FP32: weights are scaled by 2^-K
   int turn = 0;
-  for (int64_t base = int64_t(blockIdx.x) * rows; base < n; base += int64_t(gridDim.x) * rows, turn ^= 1) {
-    const int have = int(n - base < rows ? n - base : int64_t(rows));  // rows of this chunk
-    const int total = rows * d, live = have * d;
-    const T* __restrict__ xb = x + base * d;
-    T v[S::kLoads];
+  // a chunk's values and log-weights are loaded while the one before it is
+  // summed
+  T v[S::kLoads];
+  double lw = -INFINITY;
+  auto load = [&](int64_t b) {
+    const int have = int(max(int64_t(0), min(n - b, int64_t(rows))));
+    const T* __restrict__ xb = x + b * d;
 #pragma unroll
     for (int q = 0; q < S::kLoads; ++q) {
-      const int e = tid + q * kCovThreads;
-      v[q] = e < live ? xb[e] : T(0);
+      const int r = er + q * sr;
+      v[q] = (stages && r < have) ? xb[r * d + ec] : T(0);
     }
-    const double lw = tid < have ? a.logw[base + tid] : -INFINITY;
+    lw = tid < have ? a.logw[b + tid] : -INFINITY;
+  };
+  load(int64_t(blockIdx.x) * rows);
+  for (int64_t base = int64_t(blockIdx.x) * rows; base < n; base += int64_t(gridDim.x) * rows, turn ^= 1) {
+    const int have = int(n - base < rows ? n - base : int64_t(rows));  // rows of this chunk
     if constexpr (kF32) {
       float h = 0.0f, l = 0.0f;
       int E = -(1 << 20);
@@ -198,41 +220,32 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
         K = Kn;
       }
       const float f = K - E > 120 ? 0.0f : __int_as_float((127 - (K - E)) << 23);
-      s_w[tid] = h * f;
-      s_wl[tid] = l * f;
+      s_wf[tid] = make_float2(h * f, l * f);
     } else {
-      s_w[tid] = lw == -INFINITY ? 0.0 : exp(lw - m);
+      s_wd[tid] = lw == -INFINITY ? 0.0 : exp(lw - m);
     }
     __syncthreads();
-    // (opaque: the compiler would otherwise keep every value's row and column
-    // in registers from chunk to chunk, and spill)
-    int r = er, c = ec;
-    asm volatile("" : "+r"(r), "+r"(c));
 #pragma unroll
     for (int q = 0; q < S::kLoads; ++q) {
-      const int e = tid + q * kCovThreads;
-      if (e < total) {
-        const int at = r * nc + c;
+      const int r = er + q * sr;
+      if (stages && r < rows) {
+        const int at = r * nc + ec;
         if constexpr (kF32) {
-          const float rv = e < live ? centred(v[q], s_mh[c], s_ml[c]) * s_inv[c] : 0.0f;
-          const float u = __fmul_rn(s_w[r], rv);
+          const float2 w = s_wf[r];
+          const float rv = r < have ? centred(v[q], mh, ml) * inv : 0.0f;
+          const float u = __fmul_rn(w.x, rv);
           s_r[at] = rv;
           s_u[at] = u;
-          s_ul[at] = __fmaf_rn(s_wl[r], rv, __fmaf_rn(s_w[r], rv, -u));
+          s_ul[at] = __fmaf_rn(w.y, rv, __fmaf_rn(w.x, rv, -u));
         } else {
-          const double rv = e < live ? v[q] - s_mh[c] : 0.0;
+          const double rv = r < have ? v[q] - mh : 0.0;
           s_r[at] = rv;
-          s_u[at] = s_w[r] * rv;
+          s_u[at] = s_wd[r] * rv;
         }
-      }
-      r += sr;
-      c += sc;
-      if (c >= d) {
-        c -= d;
-        ++r;
       }
     }
     __syncthreads();
+    load(base + int64_t(gridDim.x) * rows);
     if (group < groups) {
 #pragma unroll 1
       for (int j = group; j < rows; j += groups) {
@@ -273,11 +286,14 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
     }
     __syncthreads();
   }
-  // the row groups' sums, added in group order, one row of every tile at a
-  // time through the space of the staged rows
+  // the row groups' sums, one row of every tile at a time through the space
+  // of the staged rows: `per` threads for each sum (as many as the block
+  // has, at most a warp) add every per-th group in order, then a fixed tree
   double* const red = reinterpret_cast<double*>(s_r);  // groups x tiles x 4 doubles
   static_assert(sizeof(s_r) >= size_t(kCovThreads) * kTileC * sizeof(double), "reduction space");
   const int npairs = d * (d + 1) / 2;
+  int per = 32;
+  while (per * tiles * kTileC > kCovThreads) per /= 2;
 #pragma unroll
   for (int p = 0; p < kTileC; ++p) {
     if (group < groups) {
@@ -287,14 +303,16 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
                                      : double(acc[p * kTileC + q]);
     }
     __syncthreads();
-    if (tid < tiles * kTileC) {
-      const int t = tid / kTileC, q = tid % kTileC;
+    const int k = tid / per, sub = tid % per;
+    double s = 0.0;
+    if (k < tiles * kTileC)
+      for (int g = sub; g < groups; g += per) s += red[g * tiles * kTileC + k];
+    for (int o = per / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (k < tiles * kTileC && sub == 0) {
       int ra, rb;
-      tile_of(t, nt, ra, rb);
-      const int ca = ra * kTileC + p, cb = rb * kTileC + q;
+      tile_of(k / kTileC, nt, ra, rb);
+      const int ca = ra * kTileC + p, cb = rb * kTileC + k % kTileC;
       if (ca <= cb && cb < d) {
-        double s = 0.0;
-        for (int g = 0; g < groups; ++g) s += red[(g * tiles + t) * kTileC + q];
         if (kF32) s = scalbn(s, K + s_ex[ca] + s_ex[cb]);
         covpart[size_t(blockIdx.x) * npairs + ca * d - ca * (ca - 1) / 2 + (cb - ca)] = s;
       }
