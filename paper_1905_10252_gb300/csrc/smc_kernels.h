@@ -31,6 +31,7 @@ struct alignas(256) TargetDev {
   const uint16_t* ximg;   // BF16 hi / lo images of X for the tensor-core likelihood
   double v[kTgtMaxD];     // X^T y in FP64
   double xsum[kTgtMaxD];  // column sums of X in FP64
+  double vw[kTgtMaxD];    // v - xsum / 2
   double prior_var;
   int32_t m;
   int32_t m_pad;          // M rounded up to the likelihood's data tile
