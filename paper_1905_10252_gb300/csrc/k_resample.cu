@@ -133,6 +133,7 @@ __global__ void k_state_init(DevState* st, int64_t n, int64_t t, int F) {
   st->pending = 0;
   st->rs_dirty = 0;
   st->rs_w = 0;
+  st->sub_ready = 0;
 }
 
 // ---------------------------------------------------------------- max of log w (stateless path)
@@ -204,6 +205,26 @@ __device__ __forceinline__ V ld_plain(const V* p) {
     return *p;
 }
 
+// eq. (7) partials of one quantise block from the move kernel's tile records
+// {M_r, sum e^{log w - M_r} x} (FP32 samplers; one warp): scaled to the units
+// of E_i (2^62 e^{log w - m}) and added over the block's tiles by a fixed
+// shuffle tree.
+__device__ __forceinline__ void quant_records(const QuantArgs& a, const int64_t blk) {
+  constexpr int kTiles = kQTile / kEstTile;
+  static_assert(kTiles <= 32, "one lane per tile record");
+  const int lane = threadIdx.x & 31, d = a.d;
+  const int64_t ntile = (a.n + kEstTile - 1) / kEstTile;
+  const int64_t jt = blk * kTiles + lane;
+  const bool have = lane < kTiles && jt < ntile && !a.st->err;
+  const double* rec = a.epart + jt * (1 + d);
+  const double Mr = have ? rec[0] : -INFINITY;
+  const float f = Mr == -INFINITY ? 0.0f : __expf(float(Mr - a.st->m)) * 0x1p62f;
+  for (int c = 0; c < d; ++c) {
+    const float v = warp_sum(have ? f * float(rec[1 + c]) : 0.0f);
+    if (lane == 0) static_cast<float*>(a.xpart)[blk * d + c] = v;
+  }
+}
+
 // Shared memory of one quantise-reduce block (declared by the calling kernel).
 struct QuantReduceSmem {
   uint64_t T[128];
@@ -218,6 +239,15 @@ __device__ __forceinline__ void quant_reduce_body(const QuantArgs& a, const int 
   double (*const shx)[32] = sm.shx;
   load_table(T);
   const DevState* st = a.st;
+  if (blk == 0 && threadIdx.x == 0) a.st->sub_ready = 0;  // (no prefixes inside the tiles from this pass)
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // rows shared by lanes (see below): 16-byte groups of kV columns
+  constexpr int kV = 16 / sizeof(ST), kLanes = DMAX / kV > 0 ? DMAX / kV : 1, kRowsPer = 32 / kLanes;
+  // (not for FP32 rows of 16: with this route the kernel needs 80 registers
+  // instead of 64, and the records route below, which these samplers take
+  // whenever they resample, 0.149 instead of 0.129 ms at N = 2^24)
+  constexpr bool kShared = EST && !COH && DMAX >= 2 * kV && !(sizeof(ST) == 4 && DMAX == 16);
+  bool shared_rows = false;
   uint64_t sw = 0;
   u128 sw2 = 0, se = 0;
   ST acc[DMAX];
@@ -295,6 +325,60 @@ __device__ __forceinline__ void quant_reduce_body(const QuantArgs& a, const int 
         done = true;
       }
     }
+    if constexpr (kShared) {
+      if (!done && !use_rec && d == DMAX) {
+        // kLanes lanes share a row, 16 bytes each, so that a warp's load covers
+        // whole 128-byte lines: the warp's 32 rows of one k come in kLanes
+        // loads of 32 / kLanes rows, lane l holding columns kV (l % kLanes) ..
+        // of rows kRowsPer j + l / kLanes, j = 0 .. kLanes - 1.  (A thread
+        // reading its own row touches 32 lines per load, kLanes times over:
+        // 54 instead of 31 us at N = 2^20, D = 32.)
+        const int lr = lane / kLanes, lc = lane % kLanes;
+        const int64_t i0 = base + (threadIdx.x - lane) + lr;  // row of (k, j): i0 + 256 k + kRows j
+        const bool whole = base + kQTile <= a.n;
+        constexpr int kUnroll = DMAX * sizeof(ST) > 128 ? 1 : 2;
+#pragma unroll kUnroll
+        for (int k = 0; k < kQItems; ++k) {
+          const int64_t i = base + k * kQThreads + threadIdx.x;
+          float4 f[kLanes];
+#pragma unroll
+          for (int j = 0; j < kLanes; ++j) {
+            const int64_t r = i0 + k * kQThreads + j * kRowsPer;
+            f[j] = (whole || r < a.n) ? ld_rows<COH>(reinterpret_cast<const float4*>(x + r * DMAX) + lc)
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+          ST w = ST(0);
+          if (i < a.n) {
+            const uint64_t E = expfx_a(__dsub_rn(m, ld_plain<COH>(a.logw + i)), T);
+            const uint64_t W = E >> sh_w;
+            a.wbuf[i] = W;
+            sw += W;
+            sw2 += u128(W) * W;
+            se += E;
+            weight_of(E, &w);
+          }
+#pragma unroll
+          for (int j = 0; j < kLanes; ++j) {
+            const ST wj = __shfl_sync(0xffffffffu, w, j * kRowsPer + lr);
+            const bool in = whole || i0 + k * kQThreads + j * kRowsPer < a.n;
+            if constexpr (sizeof(ST) == 4) {
+              const float g[4] = {f[j].x, f[j].y, f[j].z, f[j].w};
+#pragma unroll
+              for (int u = 0; u < kV; ++u)
+                if (in) acc[j * kV + u] = fma(wj, ST(g[u]), acc[j * kV + u]);
+            } else {
+              const double g[2] = {__hiloint2double(__float_as_int(f[j].y), __float_as_int(f[j].x)),
+                                   __hiloint2double(__float_as_int(f[j].w), __float_as_int(f[j].z))};
+#pragma unroll
+              for (int u = 0; u < kV; ++u)
+                if (in) acc[j * kV + u] = fma(wj, ST(g[u]), acc[j * kV + u]);
+            }
+          }
+        }
+        done = true;
+        shared_rows = true;
+      }
+    }
     if (!done)
 #pragma unroll 4
     for (int k = 0; k < kQItems; ++k) {
@@ -333,7 +417,6 @@ __device__ __forceinline__ void quant_reduce_body(const QuantArgs& a, const int 
   sw = warp_sum(sw);
   sw2 = warp_sum_u128(sw2);
   se = warp_sum_u128(se);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (lane == 0) {
     sh[wid][0] = sw;
     sh[wid][1] = uint64_t(sw2);
@@ -343,11 +426,33 @@ __device__ __forceinline__ void quant_reduce_body(const QuantArgs& a, const int 
   }
   if (EST && !use_rec) {
     // warp sums in the state precision (the FP64 pipe is scarce), then FP64
+    if (kShared && shared_rows) {
+      // the shuffle tree of warp_sum over the 32 rows (offsets 16, 8, 4, 2, 1):
+      // the high bits of a row's place are the lane's own j
+      if constexpr (kShared) {
 #pragma unroll
-    for (int c = 0; c < DMAX; ++c) {
-      if (c < d) {
-        const ST v = warp_sum(acc[c]);
-        if (lane == 0) shx[wid][c] = double(v);
+        for (int h = kLanes / 2; h > 0; h >>= 1)
+#pragma unroll
+          for (int j = 0; j < kLanes; ++j)
+            if (j < h) {
+#pragma unroll
+              for (int u = 0; u < kV; ++u) acc[j * kV + u] += acc[(j + h) * kV + u];
+            }
+#pragma unroll
+        for (int u = 0; u < kV; ++u) {
+          ST v = acc[u];
+#pragma unroll
+          for (int o = 16; o >= kLanes; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (lane < kLanes) shx[wid][lane * kV + u] = double(v);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < DMAX; ++c) {
+        if (c < d) {
+          const ST v = warp_sum(acc[c]);
+          if (lane == 0) shx[wid][c] = double(v);
+        }
       }
     }
   }
@@ -372,29 +477,226 @@ __device__ __forceinline__ void quant_reduce_body(const QuantArgs& a, const int 
     for (int w = 0; w < kQThreads / 32; ++w) v += shx[w][threadIdx.x];
     static_cast<ST*>(a.xpart)[int64_t(blk) * d + threadIdx.x] = ST(v);
   }
-  if (use_rec && wid == 0) {
-    // eq. (7) partials of this block from the move kernel's tile records
-    // {M_r, sum e^{log w - M_r} x}: scaled to the units of E_i (2^62 e^{log w - m})
-    // and added over the block's tiles by a fixed shuffle tree
-    constexpr int kTiles = kQTile / kEstTile;
-    static_assert(kTiles <= 32, "one lane per tile record");
-    const int64_t ntile = (a.n + kEstTile - 1) / kEstTile;
-    const int64_t jt = int64_t(blk) * kTiles + lane;
-    const bool have = lane < kTiles && jt < ntile && !st->err;
-    const double* rec = a.epart + jt * (1 + d);
-    const double Mr = have ? rec[0] : -INFINITY;
-    const float f = Mr == -INFINITY ? 0.0f : __expf(float(Mr - st->m)) * 0x1p62f;
-    for (int c = 0; c < d; ++c) {
-      const ST v = warp_sum(ST(have ? f * float(rec[1 + c]) : 0.0f));
-      if (lane == 0) static_cast<ST*>(a.xpart)[int64_t(blk) * d + c] = v;
-    }
-  }
+  if (use_rec && wid == 0) quant_records(a, blk);
 }
 
 template <typename ST, int DMAX, bool EST>
 __global__ void __launch_bounds__(kQThreads) k_quant_reduce(QuantArgs a) {
   __shared__ QuantReduceSmem sm;
   quant_reduce_body<ST, DMAX, EST>(a, blockIdx.x, sm);
+}
+
+// ---------------------------------------------------------------- quantise: reduce over clusters
+// The same pass for samplers of few tiles.  With one block per tile of 4096
+// weights a sampler of N = 20000 (D = 32) keeps 5 SMs busy with 16 rows per
+// thread one after another (41 us, all of it latency).  Here a cluster of
+// eight blocks shares a tile: block s quantises items [512 s, 512 s + 512)
+// and forms the eq. (7) sums of the threads 32 s .. 32 s + 31 of the one-block
+// pass (their rows: 256 k + 32 s + lane), one group of columns per warp with
+// every row load in flight; block 0 combines the eight through distributed
+// shared memory.  Every floating-point sum keeps the one-block pass's order
+// (k ascending per thread, the shuffle tree, then the warps in order), so the
+// results are the same bits.  csub receives the exclusive prefix of the
+// 512-item sums inside the tile, for a scan of 512 items per block.
+struct QuantClusterSmem {
+  uint64_t T[128];
+  uint64_t sh[kQThreads / 32][5];
+  uint64_t part[kQSplit][5];       // rank 0: the blocks' integer sums
+  double shx[kQSplit][kMaxD];      // rank 0: the blocks' column sums
+  double w[kQTile / kQSplit];      // this block's eq. (7) weights, in the state's type
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Stores v at p's place in the shared memory of the cluster's block 0.
+__device__ __forceinline__ void st_rank0(uint64_t* p, uint64_t v) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(uint32_t(__cvta_generic_to_shared(p))));
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
+}
+
+// The CW columns from c on of one row (as vectors when vec: d is a multiple
+// of CW, so that every such group is aligned and complete).
+template <int CW>
+__device__ __forceinline__ void load_cols(const float* __restrict__ row, int c, int d, bool vec, float (&v)[CW]) {
+  if (CW == 4 && vec) {
+    const float4 f = __ldg(reinterpret_cast<const float4*>(row + c));
+    v[0] = f.x;
+    v[1 % CW] = f.y;
+    v[2 % CW] = f.z;
+    v[3 % CW] = f.w;
+  } else if (CW == 2 && vec) {
+    const float2 f = __ldg(reinterpret_cast<const float2*>(row + c));
+    v[0] = f.x;
+    v[1 % CW] = f.y;
+  } else {
+#pragma unroll
+    for (int u = 0; u < CW; ++u) v[u] = c + u < d ? __ldg(row + c + u) : 0.0f;
+  }
+}
+template <int CW>
+__device__ __forceinline__ void load_cols(const double* __restrict__ row, int c, int d, bool vec, double (&v)[CW]) {
+  if (CW >= 2 && vec) {
+#pragma unroll
+    for (int u = 0; u + 1 < CW; u += 2) {
+      const double2 f = __ldg(reinterpret_cast<const double2*>(row + c + u));
+      v[u] = f.x;
+      v[u + 1] = f.y;
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < CW; ++u) v[u] = c + u < d ? __ldg(row + c + u) : 0.0;
+  }
+}
+
+template <typename ST, int CW, bool EST>
+__global__ void __launch_bounds__(kQThreads, 2) __cluster_dims__(kQSplit, 1, 1) k_quant_reduce_cluster(QuantArgs a) {
+  __shared__ QuantClusterSmem sm;
+  const int s = int(cluster_rank());
+  const int64_t tile = blockIdx.x / kQSplit;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  DevState* st = a.st;
+  const int d = a.d;
+  const int64_t n = a.n, base = tile * kQTile;
+  const bool use_rec = EST && a.est_src && st->est_ready;
+  const bool rows = EST && !use_rec;
+  const bool live = !st->err;
+  // the rows first: their loads do not wait for the weights
+  constexpr int kK = kQItems;                                     // rows per lane
+  constexpr int kG = CW * sizeof(ST) > 16 ? kK / 2 : kK;          // of them in flight
+  const int c0 = wid * CW;
+  const bool mine = rows && live && c0 < d;
+  const bool vec = d % CW == 0;
+  const ST* __restrict__ x = static_cast<const ST*>(st->cur ? a.x[1] : a.x[0]);
+  const int64_t r0 = base + 32 * s + lane;  // row of k: r0 + 256 k
+  ST xr[EST ? kG : 1][CW];
+  if constexpr (EST) {
+    if (mine) {
+#pragma unroll
+      for (int k = 0; k < kG; ++k) {
+        const int64_t i = r0 + int64_t(k) * kQThreads;
+        if (i < n) {
+          load_cols<CW>(x + i * d, c0, d, vec, xr[k]);
+        } else {
+#pragma unroll
+          for (int u = 0; u < CW; ++u) xr[k][u] = ST(0);
+        }
+      }
+    }
+  }
+  load_table(sm.T);
+  uint64_t sw = 0;
+  u128 sw2 = 0, se = 0;
+  ST* const w = reinterpret_cast<ST*>(sm.w);
+  if (live) {
+    const double m = st->m;
+    const int sh_w = 62 - st->F;
+#pragma unroll
+    for (int q = 0; q < kQTile / kQSplit / kQThreads; ++q) {
+      const int64_t i = base + s * (kQTile / kQSplit) + q * kQThreads + tid;
+      if (i < n) {
+        const uint64_t E = expfx_a(__dsub_rn(m, a.logw[i]), sm.T);
+        const uint64_t W = E >> sh_w;
+        a.wbuf[i] = W;
+        sw += W;
+        sw2 += u128(W) * W;
+        se += E;
+      }
+    }
+    if (rows) {
+#pragma unroll
+      for (int q = 0; q < kQTile / kQSplit / kQThreads; ++q) {
+        const int e = q * kQThreads + tid;  // weight of (k = e / 32, lane e % 32)
+        const int64_t i = base + int64_t(e >> 5) * kQThreads + 32 * s + (e & 31);
+        ST v = ST(0);
+        if (i < n) weight_of(expfx_a(__dsub_rn(m, a.logw[i]), sm.T), &v);
+        w[e] = v;
+      }
+    }
+  }
+  sw = warp_sum(sw);
+  sw2 = warp_sum_u128(sw2);
+  se = warp_sum_u128(se);
+  if (lane == 0) {
+    sm.sh[wid][0] = sw;
+    sm.sh[wid][1] = uint64_t(sw2);
+    sm.sh[wid][2] = uint64_t(sw2 >> 64);
+    sm.sh[wid][3] = uint64_t(se);
+    sm.sh[wid][4] = uint64_t(se >> 64);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    uint64_t tw = 0;
+    u128 t2 = 0, te = 0;
+    for (int v = 0; v < kQThreads / 32; ++v) {
+      tw += sm.sh[v][0];
+      t2 += (u128(sm.sh[v][2]) << 64) | sm.sh[v][1];
+      te += (u128(sm.sh[v][4]) << 64) | sm.sh[v][3];
+    }
+    st_rank0(&sm.part[s][0], tw);
+    st_rank0(&sm.part[s][1], uint64_t(t2));
+    st_rank0(&sm.part[s][2], uint64_t(t2 >> 64));
+    st_rank0(&sm.part[s][3], uint64_t(te));
+    st_rank0(&sm.part[s][4], uint64_t(te >> 64));
+  }
+  if constexpr (EST) {
+    if (rows && c0 < d) {
+      ST acc[CW];
+#pragma unroll
+      for (int u = 0; u < CW; ++u) acc[u] = ST(0);
+      if (live) {
+#pragma unroll
+        for (int k = 0; k < kK; ++k) {
+          if (k >= kG) {  // (wide FP64 rows: the second half, loaded as the first is used)
+            const int64_t i = r0 + int64_t(k) * kQThreads;
+            if (i < n) load_cols<CW>(x + i * d, c0, d, vec, xr[k - kG]);
+          }
+          if (r0 + int64_t(k) * kQThreads < n) {
+#pragma unroll
+            for (int u = 0; u < CW; ++u) acc[u] = fma(w[32 * k + lane], xr[k % kG][u], acc[u]);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < CW; ++u) {
+        const ST v = warp_sum(acc[u]);
+        if (lane == 0 && c0 + u < d) st_rank0(reinterpret_cast<uint64_t*>(&sm.shx[s][c0 + u]), uint64_t(__double_as_longlong(double(v))));
+      }
+    }
+  }
+  cluster_sync();
+  if (s) return;
+  if (tid == 0) {
+    uint64_t tw = 0;
+    u128 t2 = 0, te = 0;
+    for (int v = 0; v < kQSplit; ++v) {
+      a.csub[tile * kQSplit + v] = tw;
+      tw += sm.part[v][0];
+      t2 += (u128(sm.part[v][2]) << 64) | sm.part[v][1];
+      te += (u128(sm.part[v][4]) << 64) | sm.part[v][3];
+    }
+    uint64_t* q = a.qpart + 5 * tile;
+    q[0] = tw;
+    q[1] = uint64_t(t2);
+    q[2] = uint64_t(t2 >> 64);
+    q[3] = uint64_t(te);
+    q[4] = uint64_t(te >> 64);
+    if (tile == 0) st->sub_ready = 1;
+  }
+  if constexpr (EST) {
+    if (rows && tid >= 32 && tid < 32 + d) {
+      double v = 0.0;
+      for (int k = 0; k < kQSplit; ++k) v += sm.shx[k][tid - 32];
+      static_cast<ST*>(a.xpart)[tile * d + tid - 32] = ST(v);
+    }
+    if (use_rec && wid == 0) quant_records(a, tile);
+  }
 }
 
 __device__ __forceinline__ double u128_to_double(u128 v) {
@@ -660,8 +962,9 @@ struct ScanSmem {
 // kQItems for the quantise blocks of kQTile; fewer for a sampler whose N fits
 // one block of kQThreads ITEMS items (shorter per-thread chains, the same
 // exact integers).
+// base: the block's first item; C0: the exclusive prefix of W before it.
 template <int ITEMS = kQItems>
-__device__ __forceinline__ void quant_scan_body(const QuantArgs& a, const int blk, ScanSmem& sm) {
+__device__ __forceinline__ void quant_scan_body(const QuantArgs& a, const int64_t base, const uint64_t C0, ScanSmem& sm) {
   static_assert(ITEMS >= 1 && ITEMS <= kQItems, "items per thread");
   const DevState* st = a.st;
   if (st->err || !(a.force || st->flag)) return;
@@ -670,7 +973,6 @@ __device__ __forceinline__ void quant_scan_body(const QuantArgs& a, const int bl
   BigRuns& big = sm.big;
   if (threadIdx.x == 0) big.count = 0;
   const int64_t n = a.n;
-  const int64_t base = int64_t(blk) * kQTile;
   // the quantised weights of the reduce pass, staged for a blocked layout
 #pragma unroll 4
   for (int k = 0; k < ITEMS; ++k) {
@@ -688,7 +990,7 @@ __device__ __forceinline__ void quant_scan_body(const QuantArgs& a, const int bl
     tsum += W[q];
   }
   uint64_t btot;
-  uint64_t C = a.cbase[blk] + block_excl_scan_u64(tsum, scratch, &btot);
+  uint64_t C = C0 + block_excl_scan_u64(tsum, scratch, &btot);
   uint32_t ncv[ITEMS];
   unsigned nsurv = 0;
   // off_i = floor((N C_{i-1} + U) / S) for every item independently (no
@@ -781,7 +1083,27 @@ __device__ __forceinline__ void quant_scan_body(const QuantArgs& a, const int bl
 
 __global__ void __launch_bounds__(kQThreads, 4) k_quant_scan(QuantArgs a) {
   __shared__ ScanSmem sm;
-  quant_scan_body(a, blockIdx.x, sm);
+  quant_scan_body(a, int64_t(blockIdx.x) * kQTile, a.cbase[blockIdx.x], sm);
+}
+
+// 512 items per block (samplers of few tiles: eight times the blocks and two
+// quotients per thread instead of sixteen).  The prefix inside the tile comes
+// from the cluster reduce; when another reduce wrote W (a batch's), from W.
+__global__ void __launch_bounds__(kQThreads, 4) k_quant_scan_sub(QuantArgs a) {
+  constexpr int kSub = kQTile / kQSplit;
+  __shared__ ScanSmem sm;
+  const int64_t tile = blockIdx.x / kQSplit, base = int64_t(blockIdx.x) * kSub;
+  if (base >= a.n || a.st->err || !(a.force || a.st->flag)) return;
+  uint64_t C0 = a.cbase[tile];
+  if (a.st->sub_ready) {
+    C0 += a.csub[blockIdx.x];
+  } else {
+    uint64_t v = 0, total;
+    for (int64_t i = tile * kQTile + threadIdx.x; i < base; i += kQThreads) v += a.wbuf[i];
+    block_excl_scan_u64(v, sm.scratch, &total);
+    C0 += total;
+  }
+  quant_scan_body<kSub / kQThreads>(a, base, C0, sm);
 }
 
 // ---------------------------------------------------------------- standalone ncopies scan
@@ -1097,23 +1419,9 @@ __global__ void __launch_bounds__(kRThreads) k_redistribute(RedistArgs a) {
   redistribute_body<V, CPR>(a, blockIdx.x, sm);
 }
 
-// ---------------------------------------------------------------- one-block samplers
-// A sampler whose N fits one quantise block (N <= 4096) runs the reduce,
-// finalise and scan passes as one kernel of one block, with the same bodies in
-// the same order (the results are those of the three launches); one whose N
-// fits one copy tile (N <= 2048) runs redistribute and commit as one kernel.
-// For such samplers the launches, not the work, set the iteration's time.
-template <typename ST, int DMAX, bool EST>
-__global__ void __launch_bounds__(kQThreads) k_quant_small(QuantArgs a) {
-  __shared__ QuantReduceSmem sm;
-  quant_reduce_body<ST, DMAX, EST>(a, 0, sm);
-  __syncthreads();  // the block's sums, W and estimate partials are written
-  quant_finalize_body(a, 0);
-  __syncthreads();  // S, U, the decision and the block base are written
-  __shared__ ScanSmem ssm;
-  quant_scan_body(a, 0, ssm);
-}
-
+// ---------------------------------------------------------------- one-tile samplers
+// A sampler whose N fits one copy tile (N <= 2048) runs redistribute and
+// commit as one kernel.
 template <typename V, int CPR>
 __global__ void __launch_bounds__(kRThreads) k_redistribute_commit(RedistArgs a, int d, int force_flip, int recycle) {
   __shared__ RedistSmem sm;
@@ -1129,7 +1437,7 @@ __global__ void __launch_bounds__(kRThreads) k_redistribute_commit(RedistArgs a,
 // separate move launch (move_threads per block own particles); then block 0
 // alone runs, in the order of the separate launches, t += 1, the maximum, the
 // quantise reduce / finalise / scan, the copy and the commit -- the bodies of
-// k_max_finalize, k_quant_small and k_redistribute_commit -- so the results
+// k_max_finalize, k_quant_reduce / finalize / scan and k_redistribute_commit -- so the results
 // are bit for bit those of the separate launches.  At this size an iteration
 // is a chain of dependent FP64 operations (tens to thousands of cycles each
 // on this GPU) and kernel boundaries; two grid barriers per iteration replace
@@ -1219,9 +1527,9 @@ __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
       quant_finalize_body(s.q, 0);
       __syncthreads();
       if (s.a.n <= kQThreads * 4)
-        quant_scan_body<4>(s.q, 0, sm.sc);
+        quant_scan_body<4>(s.q, 0, s.q.cbase[0], sm.sc);
       else
-        quant_scan_body<8>(s.q, 0, sm.sc);
+        quant_scan_body<8>(s.q, 0, s.q.cbase[0], sm.sc);
       if (!(s.stop_last && it + 1 == s.k)) {
         __syncthreads();
         redistribute_body<V, 0, 8, true>(s.r, 0, rsm);
@@ -1293,7 +1601,7 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quant_scan_batch(const QuantAr
   const QuantArgs a = qa[m.x];
   if (m.y >= a.nblocks) return;
   __shared__ ScanSmem sm;
-  quant_scan_body(a, m.y, sm);
+  quant_scan_body(a, int64_t(m.y) * kQTile, a.cbase[m.y], sm);
 }
 
 template <int KU>
@@ -1378,19 +1686,40 @@ cudaError_t launch_max_logw(const double* logw, int64_t n, double* part, int nb,
   return cudaGetLastError();
 }
 
+// Up to kQSplitTiles = 76 tiles of 4096 weights (their eighths are at most
+// two blocks on each of 152 SMs): the cluster reduce and the scan of 512 items
+// per block.  Measured (kernel, one block per tile -> eight): reduce at 5
+// tiles, D = 32 41 -> 9.8 us; 64 tiles, D = 32 36 -> 20, FP64 D = 8 32 -> 21;
+// 17 tiles without rows 15.6 -> 5.9, its scan 14.9 -> 5.5; but 245 tiles,
+// D = 8 17 -> 28 and scan 13.0 -> 15.5 us, 4096 tiles 0.129 -> 0.50 ms (several
+// waves of blocks that each wait for the weights, their cluster and shared
+// memory of another SM).
+bool quant_split(int64_t n) { return qblocks(n) <= kQSplitTiles; }
+
 template <typename ST>
 static cudaError_t quant_reduce_t(const QuantArgs& a, cudaStream_t s) {
   const int g = qblocks(a.n);
-  if (!a.x[0] || a.d < 1)
+  const bool est = a.x[0] && a.d >= 1;
+  if (quant_split(a.n)) {
+    if (!est)
+      k_quant_reduce_cluster<ST, 1, false><<<g * kQSplit, kQThreads, 0, s>>>(a);
+    else if (a.d <= 8)
+      k_quant_reduce_cluster<ST, 1, true><<<g * kQSplit, kQThreads, 0, s>>>(a);
+    else if (a.d <= 16)
+      k_quant_reduce_cluster<ST, 2, true><<<g * kQSplit, kQThreads, 0, s>>>(a);
+    else
+      k_quant_reduce_cluster<ST, 4, true><<<g * kQSplit, kQThreads, 0, s>>>(a);
+  } else if (!est) {
     k_quant_reduce<ST, 1, false><<<g, kQThreads, 0, s>>>(a);
-  else if (a.d <= 4)
+  } else if (a.d <= 4) {
     k_quant_reduce<ST, 4, true><<<g, kQThreads, 0, s>>>(a);
-  else if (a.d <= 8)
+  } else if (a.d <= 8) {
     k_quant_reduce<ST, 8, true><<<g, kQThreads, 0, s>>>(a);
-  else if (a.d <= 16)
+  } else if (a.d <= 16) {
     k_quant_reduce<ST, 16, true><<<g, kQThreads, 0, s>>>(a);
-  else
+  } else {
     k_quant_reduce<ST, 32, true><<<g, kQThreads, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 
@@ -1404,7 +1733,10 @@ cudaError_t launch_quant_finalize(const QuantArgs& a, int set_lse_prev, cudaStre
 }
 
 cudaError_t launch_quant_scan(const QuantArgs& a, cudaStream_t s) {
-  k_quant_scan<<<qblocks(a.n), kQThreads, 0, s>>>(a);
+  if (quant_split(a.n))
+    k_quant_scan_sub<<<qblocks(a.n) * kQSplit, kQThreads, 0, s>>>(a);
+  else
+    k_quant_scan<<<qblocks(a.n), kQThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -1446,26 +1778,6 @@ cudaError_t launch_redistribute(const RedistArgs& a, cudaStream_t s) {
       k_redistribute<uint32_t, 0><<<grid, kRThreads, 0, s>>>(a);
   }
   return cudaGetLastError();
-}
-
-template <typename ST>
-static cudaError_t quant_small_t(const QuantArgs& a, cudaStream_t s) {
-  if (!a.x[0] || a.d < 1)
-    k_quant_small<ST, 1, false><<<1, kQThreads, 0, s>>>(a);
-  else if (a.d <= 4)
-    k_quant_small<ST, 4, true><<<1, kQThreads, 0, s>>>(a);
-  else if (a.d <= 8)
-    k_quant_small<ST, 8, true><<<1, kQThreads, 0, s>>>(a);
-  else if (a.d <= 16)
-    k_quant_small<ST, 16, true><<<1, kQThreads, 0, s>>>(a);
-  else
-    k_quant_small<ST, 32, true><<<1, kQThreads, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_quant_small(const QuantArgs& a, cudaStream_t s) {
-  if (qblocks(a.n) != 1) return cudaErrorInvalidValue;
-  return a.dtype == SMC_F64 ? quant_small_t<double>(a, s) : quant_small_t<float>(a, s);
 }
 
 cudaError_t launch_redistribute_commit(const RedistArgs& a, int d, int force_flip, int recycle, cudaStream_t s) {

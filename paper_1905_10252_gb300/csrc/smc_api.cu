@@ -52,6 +52,8 @@ Layout layout_for(int64_t n, int d, int m = 0, bool two_rs = false) {
   p = align_up(p + size_t(L.qblocks) * 5 * sizeof(uint64_t));
   L.cbase = p;
   p = align_up(p + size_t(L.qblocks) * sizeof(uint64_t));
+  L.csub = p;
+  if (quant_split(n)) p = align_up(p + size_t(L.qblocks) * kQSplit * sizeof(uint64_t));
   L.xpart = p;
   p = align_up(p + size_t(L.qblocks) * size_t(d < 1 ? 1 : d) * sizeof(double));
   L.rs = p;
@@ -169,6 +171,7 @@ QuantArgs quant_args(const smc_sampler* h, int force, int32_t* ncopies) {
   q.force = force;
   q.qpart = h->qpart;
   q.cbase = h->cbase;
+  q.csub = reinterpret_cast<uint64_t*>(h->ws + h->L.csub);
   q.runstart = h->rs;
   q.runstart_alt = h->rs_alt;
   q.write_rs = force ? 0 : 1;  // the fused step feeds redistribute; smc_resample does not
@@ -289,21 +292,14 @@ cudaError_t launch_iteration(smc_sampler* h, bool with_cov) {
   if (e == cudaSuccess) e = launch_max_finalize(h->part, nb, h->st, h->stream);
   QuantArgs q = quant_args(h, 0, nullptr);
   q.est_src = est_in_move(h) ? 1 : 0;
-  // (a sampler of one quantise block / one copy tile: the same bodies fused
-  // into fewer launches; the covariance reads nothing the scan writes)
-  const bool one_q = h->L.qblocks == 1, one_r = h->L.ntiles == 1;
-  if (one_q) {
-    if (e == cudaSuccess) e = launch_quant_small(q, h->stream);
-  } else {
-    if (e == cudaSuccess) e = launch_quant_reduce(q, h->stream);
-    if (e == cudaSuccess) e = launch_quant_finalize(q, 0, h->stream);
-  }
+  if (e == cudaSuccess) e = launch_quant_reduce(q, h->stream);
+  if (e == cudaSuccess) e = launch_quant_finalize(q, 0, h->stream);
   if (e == cudaSuccess && with_cov)
     e = launch_cov(a, nullptr, reinterpret_cast<double*>(h->ws + h->L.covpart), h->L.cov_blocks, h->stream);
-  if (!one_q && e == cudaSuccess) e = launch_quant_scan(q, h->stream);
+  if (e == cudaSuccess) e = launch_quant_scan(q, h->stream);
   if (h->defer) {  // the next move gathers the rows (smc_materialize, if none follows)
     if (e == cudaSuccess) e = launch_commit(h->st, h->d, 0, 1, h->stream, 1);
-  } else if (one_r) {
+  } else if (h->L.ntiles == 1) {
     if (e == cudaSuccess) e = launch_redistribute_commit(redist_args(h, 0), h->d, 0, 1, h->stream);
   } else {
     if (e == cudaSuccess) e = launch_redistribute(redist_args(h, 0), h->stream);
@@ -697,7 +693,7 @@ const char* smc_last_error(const smc_sampler* h) { return h ? h->err.c_str() : g
 // ------------------------------------------------------------------ stateless
 namespace {
 struct RawLayout {
-  size_t st, part, qpart, cbase, rs, wbuf, tile_src, stamps, total;
+  size_t st, part, qpart, cbase, csub, rs, wbuf, tile_src, stamps, total;
   int qblocks, ntiles;
 };
 RawLayout raw_layout(int64_t n) {
@@ -713,6 +709,8 @@ RawLayout raw_layout(int64_t n) {
   p = align_up(p + size_t(L.qblocks) * 5 * sizeof(uint64_t));
   L.cbase = p;
   p = align_up(p + size_t(L.qblocks) * sizeof(uint64_t));
+  L.csub = p;
+  if (quant_split(n)) p = align_up(p + size_t(L.qblocks) * kQSplit * sizeof(uint64_t));
   L.rs = p;
   p = align_up(p + size_t(n) * sizeof(int32_t));
   L.wbuf = p;
@@ -832,6 +830,7 @@ int smc_resample_raw(int64_t n, const double* logw_dev, uint64_t seed, uint64_t 
   q.force = 1;
   q.qpart = reinterpret_cast<uint64_t*>(ws + L.qpart);
   q.cbase = reinterpret_cast<uint64_t*>(ws + L.cbase);
+  q.csub = reinterpret_cast<uint64_t*>(ws + L.csub);
   q.runstart = reinterpret_cast<int32_t*>(ws + L.rs);
   q.write_rs = 0;
   q.wbuf = reinterpret_cast<uint64_t*>(ws + L.wbuf);

@@ -27,6 +27,8 @@ constexpr int kMaxD = 32;
 constexpr int kQTile = 4096;          // elements per block of the quantise / scan passes
 constexpr int kQThreads = 256;        // 16 consecutive elements per thread
 constexpr int kQItems = kQTile / kQThreads;
+constexpr int kQSplit = 8;            // blocks that share a tile in the passes of small samplers
+constexpr int kQSplitTiles = 76;       // ... of at most this many tiles
 constexpr int kRTile = 2048;          // output rows per block of the redistribute copy
 constexpr int kRThreads = 256;
 constexpr int kPThreads = 256;        // particle kernels (init / move / reweight)
@@ -65,7 +67,7 @@ struct alignas(256) DevState {
   int32_t pending;
   int32_t rs_dirty;
   int32_t rs_w;
-  int32_t rs_pad;
+  int32_t sub_ready;    // 1: csub holds the last reduce's prefixes inside the tiles (k_quant_reduce_cluster)
   double m;             // max_i log w
   double lse;           // LSE_t
   double lse_prev;      // LSE_{t-1} (0 after a reset)

@@ -100,6 +100,7 @@ struct QuantArgs {
   int32_t force;       // scan even if the decision is "no resample"
   uint64_t* qpart;     // per-block {sumW, sw2 lo, sw2 hi, sumE lo, sumE hi}
   uint64_t* cbase;     // exclusive prefix of the block sums of W
+  uint64_t* csub;      // exclusive prefix inside each block of its 512-item sums (small samplers; else NULL)
   int32_t* runstart;   // runstart[off_i] = i for every survivor (when write_rs)
   int32_t* runstart_alt;  // second run-start array (NULL: one array); st->rs_w picks
   int32_t write_rs;
@@ -239,6 +240,7 @@ cudaError_t launch_take_errors_batch(const ParticleArgs* pa, int32_t* errs, int 
 cudaError_t upload_expfx_table();  // once per device, outside stream capture
 cudaError_t expfx_table(const uint64_t** out);  // its device address (after the upload)
 cudaError_t launch_max_logw(const double* logw, int64_t n, double* part, int nb, DevState* st, cudaStream_t s);
+bool quant_split(int64_t n);  // csub is used at this size
 cudaError_t launch_quant_reduce(const QuantArgs& a, cudaStream_t s);
 cudaError_t launch_quant_finalize(const QuantArgs& a, int set_lse_prev, cudaStream_t s);
 cudaError_t launch_quant_scan(const QuantArgs& a, cudaStream_t s);
@@ -246,9 +248,7 @@ cudaError_t launch_nc_reduce(const NcScanArgs& a, cudaStream_t s);
 cudaError_t launch_nc_finalize(const NcScanArgs& a, cudaStream_t s);
 cudaError_t launch_nc_scan(const NcScanArgs& a, cudaStream_t s);
 cudaError_t launch_redistribute(const RedistArgs& a, cudaStream_t s);
-// one-block samplers: quantise reduce + finalise + scan (N <= 4096), and
-// redistribute + commit (N <= 2048), each as one launch
-cudaError_t launch_quant_small(const QuantArgs& a, cudaStream_t s);
+// one-tile samplers (N <= 2048): redistribute + commit as one launch
 cudaError_t launch_redistribute_commit(const RedistArgs& a, int d, int force_flip, int recycle, cudaStream_t s);
 
 // k iterations of an FP64 sampler of one quantise block and one copy tile
