@@ -579,8 +579,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_logistic_tc(ParticleArgs a) {
       v = wmax[w] > v ? wmax[w] : v;
       nan |= wnan[w];
     }
-    a.part[2 * blockIdx.x] = from_ordered_key(v);
-    a.part[2 * blockIdx.x + 1] = 1.0;
+    if (a.flags & PA_FUSED_ITER) {
+      atomicMax(&a.st->mkey, v);
+    } else {
+      a.part[2 * blockIdx.x] = from_ordered_key(v);
+      a.part[2 * blockIdx.x + 1] = 1.0;
+    }
     if (nan) record_error(a.st, SMC_ENONFINITE);
     if (*abort_flag) record_error(a.st, SMC_ETIMEOUT);
   }

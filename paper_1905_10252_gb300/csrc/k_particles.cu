@@ -197,7 +197,8 @@ __global__ void __launch_bounds__(kPThreads) k_init(ParticleArgs a) {
 template <typename T, int DMAX, bool MOVE, bool REWEIGHT>
 __global__ void __launch_bounds__(kPThreads) k_move_reweight(ParticleArgs a) {
   __shared__ TargetSmem<T> ts;
-  move_reweight_generic_body<T, DMAX, MOVE, REWEIGHT>(a, ts, blockIdx.x, gridDim.x, blockDim.x, 0);
+  move_reweight_generic_body<T, DMAX, MOVE, REWEIGHT>(a, ts, blockIdx.x, gridDim.x, blockDim.x,
+                                                      (a.flags & PA_FUSED_ITER) ? 1 : 0);
 }
 
 // ---------------------------------------------------------------- move + reweight, FP32 fast path
@@ -493,7 +494,7 @@ __device__ __forceinline__ void move_reweight_body(const ParticleArgs& a, const 
 #pragma unroll
   for (int c = 0; c < (EST ? DMAX : 1); ++c) eacc[c] = 0.0f;
   const int cur = a.st->cur;
-  const uint64_t t = uint64_t(a.st->t);
+  const uint64_t t = uint64_t(a.st->t + ((a.flags & PA_FUSED_ITER) ? 1 : 0));
   float* __restrict__ x = static_cast<float*>(cur ? a.x[1] : a.x[0]);
   float* __restrict__ lp = static_cast<float*>(cur ? a.logpi[1] : a.logpi[0]);
   double* __restrict__ logw = a.logw;
@@ -711,7 +712,7 @@ __device__ __forceinline__ void move_reweight_body(const ParticleArgs& a, const 
       mt.add(R + double(__int_as_float(b)));
       mt.nan = mt.nan || dnan;
     }
-    block_write_max(mt, a.part + 2 * blk, a.st);
+    block_write_max(mt, a.part + 2 * blk, a.st, a.flags & PA_FUSED_ITER);
   }
 }
 

@@ -134,6 +134,8 @@ __global__ void k_state_init(DevState* st, int64_t n, int64_t t, int F) {
   st->rs_dirty = 0;
   st->rs_w = 0;
   st->sub_ready = 0;
+  st->mkey = kNoMaxKey;
+  st->tickets = 0;
 }
 
 // ---------------------------------------------------------------- max of log w (stateless path)
@@ -187,6 +189,21 @@ __device__ __forceinline__ float u64_to_float_trunc(uint64_t v) {
 __device__ __forceinline__ void weight_of(uint64_t E, float* w) { *w = u64_to_float_trunc(E); }
 __device__ __forceinline__ void weight_of(uint64_t E, double* w) { *w = __ull2double_rn(E); }
 
+// What a quantise pass starts from.  In smc_step's own iteration no kernel has
+// run between the move and this pass: the maximum is still a key, a move that
+// gathered a pending copy wrote the other buffer, and the eq. (7) records
+// are there when the weights started uniform (k_iter_finalize then brings the
+// state up to date).
+__device__ __forceinline__ double pass_max(const QuantArgs& a) {
+  return a.fused ? from_ordered_key(a.st->mkey) : a.st->m;
+}
+__device__ __forceinline__ bool pass_cur(const QuantArgs& a) {
+  return a.fused ? (a.st->cur ^ a.st->pending) != 0 : a.st->cur != 0;
+}
+__device__ __forceinline__ bool pass_records(const QuantArgs& a) {
+  return a.est_src && (a.fused ? a.st->w_uniform : a.st->est_ready);
+}
+
 // Loads of rows the kernel only reads (read-only path), or, in a kernel whose
 // other blocks wrote them before a grid barrier, at the coherent level (L2).
 template <bool COH, typename V>
@@ -218,7 +235,7 @@ __device__ __forceinline__ void quant_records(const QuantArgs& a, const int64_t 
   const bool have = lane < kTiles && jt < ntile && !a.st->err;
   const double* rec = a.epart + jt * (1 + d);
   const double Mr = have ? rec[0] : -INFINITY;
-  const float f = Mr == -INFINITY ? 0.0f : __expf(float(Mr - a.st->m)) * 0x1p62f;
+  const float f = Mr == -INFINITY ? 0.0f : __expf(float(Mr - pass_max(a))) * 0x1p62f;
   for (int c = 0; c < d; ++c) {
     const float v = warp_sum(have ? f * float(rec[1 + c]) : 0.0f);
     if (lane == 0) static_cast<float*>(a.xpart)[blk * d + c] = v;
@@ -256,12 +273,12 @@ __device__ __forceinline__ void quant_reduce_body(const QuantArgs& a, const int 
   const int d = a.d;
   // eq. (7) from the move kernel's tile records when it wrote them this
   // iteration, else from the rows
-  const bool use_rec = EST && a.est_src && st->est_ready;
+  const bool use_rec = EST && pass_records(a);
   if (!st->err) {
-    const double m = st->m;
+    const double m = pass_max(a);
     const int sh_w = 62 - st->F;
     const int64_t base = int64_t(blk) * kQTile;
-    const ST* __restrict__ x = static_cast<const ST*>(st->cur ? a.x[1] : a.x[0]);
+    const ST* __restrict__ x = static_cast<const ST*>(pass_cur(a) ? a.x[1] : a.x[0]);
     bool done = false;
     if constexpr (sizeof(ST) == 4) {  // (records exist for FP32 samplers only)
       if (use_rec) {
@@ -564,7 +581,7 @@ __global__ void __launch_bounds__(kQThreads, 2) __cluster_dims__(kQSplit, 1, 1) 
   DevState* st = a.st;
   const int d = a.d;
   const int64_t n = a.n, base = tile * kQTile;
-  const bool use_rec = EST && a.est_src && st->est_ready;
+  const bool use_rec = EST && pass_records(a);
   const bool rows = EST && !use_rec;
   const bool live = !st->err;
   // the rows first: their loads do not wait for the weights
@@ -573,7 +590,7 @@ __global__ void __launch_bounds__(kQThreads, 2) __cluster_dims__(kQSplit, 1, 1) 
   const int c0 = wid * CW;
   const bool mine = rows && live && c0 < d;
   const bool vec = d % CW == 0;
-  const ST* __restrict__ x = static_cast<const ST*>(st->cur ? a.x[1] : a.x[0]);
+  const ST* __restrict__ x = static_cast<const ST*>(pass_cur(a) ? a.x[1] : a.x[0]);
   const int64_t r0 = base + 32 * s + lane;  // row of k: r0 + 256 k
   ST xr[EST ? kG : 1][CW];
   if constexpr (EST) {
@@ -595,7 +612,7 @@ __global__ void __launch_bounds__(kQThreads, 2) __cluster_dims__(kQSplit, 1, 1) 
   u128 sw2 = 0, se = 0;
   ST* const w = reinterpret_cast<ST*>(sm.w);
   if (live) {
-    const double m = st->m;
+    const double m = pass_max(a);
     const int sh_w = 62 - st->F;
 #pragma unroll
     for (int q = 0; q < kQTile / kQSplit / kQThreads; ++q) {
@@ -703,6 +720,67 @@ __device__ __forceinline__ double u128_to_double(u128 v) {
   return double(uint64_t(v >> 64)) * 0x1p64 + double(uint64_t(v));
 }
 
+// eq. (7)'s numerators sum_i E_i x_i from the per-block partial sums, into
+// sxsum[kMaxD] (shared memory); the whole block takes part.
+__device__ __forceinline__ void estimate_sums(const QuantArgs& a, double* tpart, double* sxsum) {
+  const int nb = a.nblocks;
+  // logical thread j (of kFinThreads, whatever the block size) sums column
+  // j % d over rows j / d, j / d + stride / d, ... in a fixed order
+  // (deterministic, and the same in one-sampler and batched launches), in
+  // the particle precision (the FP64 pipe is scarce); the per-thread
+  // partials are then added in order per column
+  const int stride = (kFinThreads / a.d) * a.d;
+  const int64_t total_words = int64_t(nb) * a.d;
+  for (int lt = threadIdx.x; lt < kFinThreads; lt += blockDim.x) {
+    double part = 0.0;
+    if (lt < stride) {
+      if (a.dtype == SMC_F64) {
+        const double* xp = static_cast<const double*>(a.xpart);
+        for (int64_t j = lt; j < total_words; j += stride) part += xp[j];
+      } else {
+        const float* xp = static_cast<const float*>(a.xpart);
+        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        int64_t j = lt;
+        const int64_t s1 = int64_t(stride), s8 = 8 * s1;
+        // four rounds' loads in flight at once, then their additions in
+        // round order (the same sums as one round at a time)
+        for (; j + 3 * s8 + 7 * s1 < total_words; j += 4 * s8) {
+          float tv[32];
+#pragma unroll
+          for (int r = 0; r < 32; ++r) tv[r] = xp[j + r * s1];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] += tv[8 * q + u];
+        }
+        for (; j + 7 * s1 < total_words; j += s8) {
+#pragma unroll
+          for (int u = 0; u < 8; ++u) v[u] += xp[j + u * s1];
+        }
+        for (; j < total_words; j += stride) v[0] += xp[j];
+        part = double(((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])));
+      }
+    }
+    tpart[lt] = part;
+  }
+  __syncthreads();
+  // column c's stride / d partials (tpart[c + d j]) summed by warps
+  // c, c + nw, ...: lane l adds j = l, l + 32, ... in order, then a fixed
+  // shuffle tree -- deterministic, and a short FP64 dependency chain
+  {
+    const int per_col = stride / a.d;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    for (int c = wid; c < a.d; c += nwarps) {
+      double t = 0.0;
+      for (int j = lane; j < per_col; j += 32) t += tpart[c + a.d * j];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) sxsum[c] = t;
+    }
+  }
+  __syncthreads();
+}
+
 // ---------------------------------------------------------------- quantise: finalise
 // Single block: totals, exclusive prefix of the block sums (the CDF base of
 // each scan block), decision, systematic offset U, division constants, LSE,
@@ -748,62 +826,8 @@ __device__ __forceinline__ void quant_finalize_body(const QuantArgs& a, const in
   __shared__ double sxsum[kMaxD];
   const bool est = a.x[0] != nullptr && a.d > 0;
   if (est) {
-    // logical thread j (of kFinThreads, whatever the block size) sums column
-    // j % d over rows j / d, j / d + stride / d, ... in a fixed order
-    // (deterministic, and the same in one-sampler and batched launches), in
-    // the particle precision (the FP64 pipe is scarce); the per-thread
-    // partials are then added in order per column
-    const int stride = (kFinThreads / a.d) * a.d;
-    const int64_t total_words = int64_t(nb) * a.d;
     __shared__ double tpart[kFinThreads];
-    for (int lt = threadIdx.x; lt < kFinThreads; lt += blockDim.x) {
-      double part = 0.0;
-      if (lt < stride) {
-        if (a.dtype == SMC_F64) {
-          const double* xp = static_cast<const double*>(a.xpart);
-          for (int64_t j = lt; j < total_words; j += stride) part += xp[j];
-        } else {
-          const float* xp = static_cast<const float*>(a.xpart);
-          float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-          int64_t j = lt;
-          const int64_t s1 = int64_t(stride), s8 = 8 * s1;
-          // four rounds' loads in flight at once, then their additions in
-          // round order (the same sums as one round at a time)
-          for (; j + 3 * s8 + 7 * s1 < total_words; j += 4 * s8) {
-            float tv[32];
-#pragma unroll
-            for (int r = 0; r < 32; ++r) tv[r] = xp[j + r * s1];
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-              for (int u = 0; u < 8; ++u) v[u] += tv[8 * q + u];
-          }
-          for (; j + 7 * s1 < total_words; j += s8) {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] += xp[j + u * s1];
-          }
-          for (; j < total_words; j += stride) v[0] += xp[j];
-          part = double(((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])));
-        }
-      }
-      tpart[lt] = part;
-    }
-    __syncthreads();
-    // column c's stride / d partials (tpart[c + d j]) summed by warps
-    // c, c + nw, ...: lane l adds j = l, l + 32, ... in order, then a fixed
-    // shuffle tree -- deterministic, and a short FP64 dependency chain
-    {
-      const int per_col = stride / a.d;
-      const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-      for (int c = wid; c < a.d; c += nwarps) {
-        double t = 0.0;
-        for (int j = lane; j < per_col; j += 32) t += tpart[c + a.d * j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) sxsum[c] = t;
-      }
-    }
-    __syncthreads();
+    estimate_sums(a, tpart, sxsum);
   }
   // eq. (7): the weighted mean, one column per thread
   {
@@ -903,6 +927,230 @@ __device__ __forceinline__ void quant_finalize_body(const QuantArgs& a, const in
 
 __global__ void __launch_bounds__(kFinThreads) k_quant_finalize(QuantArgs a, int set_lse_prev) {
   quant_finalize_body(a, set_lse_prev);
+}
+
+// ---------------------------------------------------------------- an iteration of smc_step: finalise
+// The single-block part that the scan waits for, and nothing else: the
+// totals, the CDF base of every block, the decision, U and floor(N 2^64 / S),
+// and the state's step from t - 1 to t.  What only the caller reads (LSE,
+// N_eff, the mean, the recycling sums) is the scan launch's extra block
+// (iter_stats), off the chain of kernels.  As begin + maximum + finalise + commit
+// kernels, with the logarithm and divisions of the statistics in the chain,
+// these steps took 22 us of an iteration whatever N.
+__global__ void __launch_bounds__(kFinThreads) k_iter_finalize(QuantArgs a) {
+  __shared__ uint64_t s_w[33], s_2l[32], s_2h[32], s_el[32], s_eh[32];
+  DevState* st = a.st;
+  const int nb = a.nblocks, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+  // (each of the four threads at work in the end loads what it needs now)
+  const bool role = lane == 0 && wid < 4;
+  int wu = 0, pend = 0, cur = 0, rsw = 0, err = 0;
+  int64_t t = 0, t0 = 0;
+  long long key = 0;
+  smc_iter_stats* trace = nullptr;
+  if (role) {
+    err = st->err;
+    key = st->mkey;
+    t = st->t + 1;
+    if (wid == 3) {
+      wu = st->w_uniform;
+      pend = st->pending;
+      cur = st->cur;
+      rsw = st->rs_w;
+      trace = st->trace;
+      t0 = st->trace_t0;
+    }
+  }
+  const int chunk = (nb + blockDim.x - 1) / blockDim.x;
+  const int b0 = tid * chunk, b1 = min(nb, b0 + chunk);
+  uint64_t tw = 0;
+  u128 t2 = 0, te = 0;
+#pragma unroll 4
+  for (int b = b0; b < b1; ++b) {
+    const uint64_t* q = a.qpart + 5 * int64_t(b);
+    tw += q[0];
+    t2 += (u128(q[2]) << 64) | q[1];
+    te += (u128(q[4]) << 64) | q[3];
+  }
+  const uint64_t incl = warp_incl_scan_u64(tw);
+  t2 = warp_sum_u128(t2);
+  te = warp_sum_u128(te);
+  if (lane == 31) s_w[wid] = incl;
+  if (lane == 0) {
+    s_2l[wid] = uint64_t(t2);
+    s_2h[wid] = uint64_t(t2 >> 64);
+    s_el[wid] = uint64_t(te);
+    s_eh[wid] = uint64_t(te >> 64);
+  }
+  __syncthreads();
+  uint64_t S = 0, pre = 0;  // every warp adds up the warps' totals it needs
+  {
+    const uint64_t v = lane < nw ? s_w[lane] : 0;
+    const uint64_t vi = warp_incl_scan_u64(v);
+    S = __shfl_sync(0xffffffffu, vi, 31);
+    pre = __shfl_sync(0xffffffffu, vi - v, wid);
+  }
+  pre += incl - tw;
+  for (int b = b0; b < b1; ++b) {
+    a.cbase[b] = pre;
+    pre += a.qpart[5 * int64_t(b)];
+  }
+  if (wid >= 4) return;
+  u128 sw2 = 0, se = 0;
+  if (wid == 1) sw2 = warp_sum_u128(lane < nw ? (u128(s_2h[lane]) << 64) | s_2l[lane] : u128(0));
+  if (wid == 2) se = warp_sum_u128(lane < nw ? (u128(s_eh[lane]) << 64) | s_el[lane] : u128(0));
+  if (!role) return;
+  const double M = from_ordered_key(key);
+  const bool bad = !(M > -INFINITY && M < INFINITY);
+  const uint64_t n = uint64_t(a.n);
+  if (wid == 0) {
+    st->S = S;
+    st->recip = S > n ? quotient_2p64(n, S) : 0;  // (S > N unless an error left no weight)
+  } else if (wid == 1) {
+    int flag = 0;
+    if (!err && !bad && S > 0) {
+      if (a.mode == SMC_RESAMPLE_ALWAYS)
+        flag = 1;
+      else if (a.mode == SMC_RESAMPLE_NEVER)
+        flag = 0;
+      else if (a.nstar > 0)  // N_eff < N*  <=>  S^2 < N* sum W^2 (Algorithm 2, line 7)
+        flag = u128(S) * S < u128(uint64_t(a.nstar)) * sw2;
+      else  // N* = N/2
+        flag = (u128(S) * S * 2) < u128(n) * sw2;
+    }
+    st->flag = flag;
+    st->sw2_lo = uint64_t(sw2);
+    st->sw2_hi = uint64_t(sw2 >> 64);
+  } else if (wid == 2) {
+    const P4 r = stream_block(a.seed, uint64_t(t), kPurposeResample, 0xFFFFFFFFull, 0);
+    const uint64_t r64 = (uint64_t(r.v[0]) << 32) | r.v[1];
+    st->U = S ? __umul64hi(r64, S) : 0;
+    st->L = S ? 64 - __clzll((long long)S) : 1;
+    st->se_lo = uint64_t(se);
+    st->se_hi = uint64_t(se >> 64);
+  } else {
+    if (bad) record_error(st, SMC_ENONFINITE);
+    st->t = t;
+    st->m = M;
+    st->mkey = kNoMaxKey;
+    // the move wrote eq. (7) records iff the weights it started from were
+    // uniform; after its reweight they are not
+    st->est_ready = wu;
+    st->w_uniform = 0;
+    // a move that gathered a deferred resampling's rows wrote them to the
+    // other buffer, which is now current; the run starts it read stay set, so
+    // the next scan writes the other array (which that move reset if it was
+    // dirty) and this one is marked dirty
+    if (pend) {
+      st->cur = cur ^ 1;
+      st->pending = 0;
+      st->rs_w = rsw ^ 1;
+      st->rs_dirty = 1;
+    }
+    st->survivors = 0;
+    st->last.survivors = 0;
+    if (trace && t - t0 - 1 >= 0) trace[t - t0 - 1].survivors = 0;
+  }
+}
+
+// The iteration's statistics (one block, beside the scan's): LSE, N_eff, log
+// c_t, the mean of eq. (7) and the recycling sums of eq. (6), each with the
+// operations of quant_finalize_body and commit_warp in their order.
+struct IterStatsSmem {
+  double tpart[kFinThreads];
+  double sxsum[kMaxD];
+  double lse, ess;
+};
+__device__ __forceinline__ void iter_stats(const QuantArgs& a, IterStatsSmem& sm) {
+  DevState* st = a.st;
+  const int tid = threadIdx.x, last_warp = (blockDim.x >> 5) - 1;
+  const double se_d = u128_to_double((u128(st->se_hi) << 64) | st->se_lo);
+  // the two longest chains first, on warps of their own
+  if (tid == 32 * last_warp) sm.lse = st->m + log(se_d * 0x1p-62);
+  if (tid == 32 * (last_warp - 1)) {
+    const double Sd = double(st->S);
+    const u128 sw2 = (u128(st->sw2_hi) << 64) | st->sw2_lo;
+    sm.ess = (st->S && sw2) ? Sd * Sd / u128_to_double(sw2) : 0.0;
+  }
+  const bool est = a.x[0] != nullptr && a.d > 0;
+  if (est)
+    estimate_sums(a, sm.tpart, sm.sxsum);
+  else
+    __syncthreads();
+  if (tid >= 32) return;
+  const int err = st->err, flag = st->flag;
+  const int64_t t = st->t, t0 = st->trace_t0;
+  const double m = st->m, lse_prev = st->lse_prev, rmax = st->rc_max, rden = st->rc_den;
+  smc_iter_stats* const trace = st->trace;
+  double* const fh = st->fhat_out;
+  double* const mean_out = st->mean_out;
+  const double lse = sm.lse, logc = lse - lse_prev;
+  static_assert(kMaxD <= 32, "one column per lane");
+  if (est && !err) {
+    double mc = 0.0, rnum = 0.0;
+    if (tid < a.d) {
+      rnum = st->rc_num[tid];
+      mc = se_d > 0.0 ? sm.sxsum[tid] / se_d : st->mean[tid];
+    }
+    const double M = fmax(rmax, logc);
+    const double sc = (rmax == -INFINITY) ? 0.0 : exp(__dsub_rn(rmax, M));
+    const double e = exp(__dsub_rn(logc, M));
+    const double den = __fma_rn(rden, sc, e);
+    if (tid < a.d) {
+      st->mean[tid] = mc;
+      if (mean_out) mean_out[tid] = mc;
+      const double num = __fma_rn(rnum, sc, __dmul_rn(e, mc));
+      st->rc_num[tid] = num;
+      if (fh) fh[tid] = __ddiv_rn(num, den);
+    }
+    __syncwarp();  // (every lane has read the sums' scale)
+    if (tid == 0) {
+      st->rc_den = den;
+      st->rc_max = M;
+    }
+  }
+  if (tid) return;
+  st->est_s = se_d * 0x1p-62;
+  st->lse = lse;
+  st->ess = sm.ess;
+  st->logc = logc;
+  // LSE_t becomes the next LSE_{t-1}, 0 after a reset
+  st->lse_prev = (flag && !err) ? 0.0 : lse;
+  // (survivors: the finaliser zeroed it, the end of the iteration sets it)
+  const int64_t idx = t - t0 - 1;
+  smc_iter_stats* const recs[2] = {&st->last, trace && idx >= 0 ? trace + idx : nullptr};
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    if (!recs[k]) continue;
+    recs[k]->lse = lse;
+    recs[k]->logc = logc;
+    recs[k]->ess = sm.ess;
+    recs[k]->max_logw = m;
+    recs[k]->resampled = flag;
+    recs[k]->t = t;
+  }
+}
+
+// The end of an iteration, by the last block of its last kernel to finish (so
+// that every block has read the state it changes): a resampled iteration's
+// copy becomes current, or pending when the next move makes it.  All threads
+// of every block call it once.
+__device__ __forceinline__ void end_iteration(DevState* st, unsigned blocks, int defer) {
+  __syncthreads();
+  if (threadIdx.x) return;
+  __threadfence();
+  if (atomicAdd(&st->tickets, 1u) != blocks - 1) return;
+  __threadfence();
+  st->tickets = 0;
+  if (!st->flag || st->err) return;
+  const int64_t surv = int64_t(*const_cast<volatile unsigned long long*>(&st->survivors));
+  st->last.survivors = surv;
+  const int64_t idx = st->t - st->trace_t0 - 1;
+  if (st->trace && idx >= 0) st->trace[idx].survivors = surv;
+  st->w_uniform = 1;  // a resampled iteration leaves every log w at reset_logw
+  if (defer)
+    st->pending = 1;
+  else
+    st->cur ^= 1;
 }
 
 // ---------------------------------------------------------------- copy-tile sources
@@ -1104,6 +1352,29 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quant_scan_sub(QuantArgs a) {
     C0 += total;
   }
   quant_scan_body<kSub / kQThreads>(a, base, C0, sm);
+}
+
+// The scan of an iteration of smc_step (SUB: 512 items per block), its
+// statistics in the first block (so that they run beside the scan, not after
+// it: as the last block they ended a scan of 4096 blocks 10 us later).
+template <bool SUB>
+__global__ void __launch_bounds__(kQThreads, 4) k_iter_scan(QuantArgs a) {
+  __shared__ union {
+    ScanSmem scan;
+    IterStatsSmem stats;
+  } sm;
+  const int blk = int(blockIdx.x) - 1;
+  if (blk < 0) {
+    iter_stats(a, sm.stats);
+  } else if constexpr (SUB) {
+    constexpr int kSub = kQTile / kQSplit;
+    const int64_t base = int64_t(blk) * kSub;
+    if (base < a.n && !a.st->err && a.st->flag)
+      quant_scan_body<kSub / kQThreads>(a, base, a.cbase[blk / kQSplit] + a.csub[blk], sm.scan);
+  } else {
+    quant_scan_body(a, int64_t(blk) * kQTile, a.cbase[blk], sm.scan);
+  }
+  if (a.defer) end_iteration(a.st, gridDim.x, 1);
 }
 
 // ---------------------------------------------------------------- standalone ncopies scan
@@ -1417,6 +1688,7 @@ template <typename V, int CPR>
 __global__ void __launch_bounds__(kRThreads) k_redistribute(RedistArgs a) {
   __shared__ RedistSmem sm;
   redistribute_body<V, CPR>(a, blockIdx.x, sm);
+  if (a.end_iter) end_iteration(a.st, gridDim.x, 0);
 }
 
 // ---------------------------------------------------------------- one-tile samplers
@@ -1737,6 +2009,19 @@ cudaError_t launch_quant_scan(const QuantArgs& a, cudaStream_t s) {
     k_quant_scan_sub<<<qblocks(a.n) * kQSplit, kQThreads, 0, s>>>(a);
   else
     k_quant_scan<<<qblocks(a.n), kQThreads, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_iter_finalize(const QuantArgs& a, cudaStream_t s) {
+  k_iter_finalize<<<1, a.nblocks > 256 ? kFinThreads : 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_iter_scan(const QuantArgs& a, cudaStream_t s) {
+  if (quant_split(a.n))
+    k_iter_scan<true><<<qblocks(a.n) * kQSplit + 1, kQThreads, 0, s>>>(a);
+  else
+    k_iter_scan<false><<<qblocks(a.n) + 1, kQThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 

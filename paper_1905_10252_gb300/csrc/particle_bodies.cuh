@@ -136,8 +136,10 @@ __device__ __forceinline__ void store_row(T* __restrict__ p, int d, const T (&x)
   }
 }
 
-// One record per block: rec[0] = max log w of the block, rec[1] = 1.
-__device__ __forceinline__ void block_write_max(const MaxTracker& mt, double* __restrict__ rec, DevState* st) {
+// One record per block: rec[0] = max log w of the block, rec[1] = 1; in an
+// iteration of smc_step the block raises st->mkey instead.
+__device__ __forceinline__ void block_write_max(const MaxTracker& mt, double* __restrict__ rec, DevState* st,
+                                                bool fused = false) {
   __shared__ long long shm[kPThreads / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   if (mt.nan) record_error(st, SMC_ENONFINITE);
@@ -147,8 +149,12 @@ __device__ __forceinline__ void block_write_max(const MaxTracker& mt, double* __
   if (threadIdx.x == 0) {
     long long v = shm[0];
     for (int w = 1; w < nw; ++w) v = shm[w] > v ? shm[w] : v;
-    rec[0] = from_ordered_key(v);
-    rec[1] = 1.0;
+    if (fused) {
+      atomicMax(&st->mkey, v);
+    } else {
+      rec[0] = from_ordered_key(v);
+      rec[1] = 1.0;
+    }
   }
 }
 
@@ -235,7 +241,7 @@ __device__ __forceinline__ void move_reweight_generic_body(const ParticleArgs& a
       mt.add(lw);
     }
   }
-  if (REWEIGHT) block_write_max(mt, a.part + 2 * blk, a.st);
+  if (REWEIGHT) block_write_max(mt, a.part + 2 * blk, a.st, a.flags & PA_FUSED_ITER);
 }
 
 // ---------------------------------------------------------------- finalise the maximum

@@ -283,28 +283,37 @@ cudaError_t launch_move_reweight(smc_sampler* h, const ParticleArgs& a, int* nb)
   return launch_particles(op, a, h->grid_p, h->threads_p, h->stream, gauss_params(h));
 }
 
-// One iteration of Algorithm 2 (lines 3-10), all on h->stream.
-cudaError_t launch_iteration(smc_sampler* h, bool with_cov) {
-  const ParticleArgs a = particle_args(h);
-  int nb = 0;
-  cudaError_t e = launch_begin(h->st, h->stream);
-  if (e == cudaSuccess) e = launch_move_reweight(h, a, &nb);
-  if (e == cudaSuccess) e = launch_max_finalize(h->part, nb, h->st, h->stream);
+QuantArgs iter_quant_args(const smc_sampler* h) {
   QuantArgs q = quant_args(h, 0, nullptr);
   q.est_src = est_in_move(h) ? 1 : 0;
+  q.fused = 1;
+  q.defer = h->defer ? 1 : 0;
+  return q;
+}
+
+// Algorithm 5 of an iteration, which it ends.
+RedistArgs iter_redist_args(const smc_sampler* h) {
+  RedistArgs r = redist_args(h, 0);
+  r.end_iter = 1;
+  return r;
+}
+
+// One iteration of Algorithm 2 (lines 3-10), all on h->stream: five kernels
+// (four when the next move makes the copy), each ordered after the one before.
+// (The covariance reads nothing the scan writes, and the mean that its extra
+// block forms.)
+cudaError_t launch_iteration(smc_sampler* h, bool with_cov) {
+  ParticleArgs a = particle_args(h);
+  a.flags |= PA_FUSED_ITER;
+  int nb = 0;
+  const QuantArgs q = iter_quant_args(h);
+  cudaError_t e = launch_move_reweight(h, a, &nb);
   if (e == cudaSuccess) e = launch_quant_reduce(q, h->stream);
-  if (e == cudaSuccess) e = launch_quant_finalize(q, 0, h->stream);
+  if (e == cudaSuccess) e = launch_iter_finalize(q, h->stream);
+  if (e == cudaSuccess) e = launch_iter_scan(q, h->stream);
   if (e == cudaSuccess && with_cov)
     e = launch_cov(a, nullptr, reinterpret_cast<double*>(h->ws + h->L.covpart), h->L.cov_blocks, h->stream);
-  if (e == cudaSuccess) e = launch_quant_scan(q, h->stream);
-  if (h->defer) {  // the next move gathers the rows (smc_materialize, if none follows)
-    if (e == cudaSuccess) e = launch_commit(h->st, h->d, 0, 1, h->stream, 1);
-  } else if (h->L.ntiles == 1) {
-    if (e == cudaSuccess) e = launch_redistribute_commit(redist_args(h, 0), h->d, 0, 1, h->stream);
-  } else {
-    if (e == cudaSuccess) e = launch_redistribute(redist_args(h, 0), h->stream);
-    if (e == cudaSuccess) e = launch_commit(h->st, h->d, 0, 1, h->stream);
-  }
+  if (e == cudaSuccess && !h->defer) e = launch_redistribute(iter_redist_args(h), h->stream);
   return e;
 }
 
@@ -599,20 +608,18 @@ int smc_step_profile(smc_sampler* h, double* mean_dev, void* const* events_host,
   };
   SMC_TRY(h, fetch_gp(h));
   SMC_TRY(h, launch_step_setup(h->st, nullptr, mean_dev, nullptr, nullptr, s));
-  const ParticleArgs a = particle_args(h);
-  QuantArgs q = quant_args(h, 0, nullptr);
-  q.est_src = est_in_move(h) ? 1 : 0;
+  ParticleArgs a = particle_args(h);
+  a.flags |= PA_FUSED_ITER;
+  const QuantArgs q = iter_quant_args(h);
   int nb = 0;
   SMC_TRY(h, rec(0));
   {
     SMC_RANGE("move+reweight");
-    SMC_TRY(h, launch_begin(h->st, s));
     SMC_TRY(h, launch_move_reweight(h, a, &nb));
   }
   SMC_TRY(h, rec(1));
   {
-    SMC_RANGE("max finalise");
-    SMC_TRY(h, launch_max_finalize(h->part, nb, h->st, s));
+    SMC_RANGE("max finalise");  // (part of the move and of the finaliser)
   }
   SMC_TRY(h, rec(2));
   {
@@ -622,22 +629,21 @@ int smc_step_profile(smc_sampler* h, double* mean_dev, void* const* events_host,
   SMC_TRY(h, rec(3));
   {
     SMC_RANGE("quantise finalise");
-    SMC_TRY(h, launch_quant_finalize(q, 0, s));
+    SMC_TRY(h, launch_iter_finalize(q, s));
   }
   SMC_TRY(h, rec(4));
   {
     SMC_RANGE("systematic scan");
-    SMC_TRY(h, launch_quant_scan(q, s));
+    SMC_TRY(h, launch_iter_scan(q, s));
   }
   SMC_TRY(h, rec(5));
   if (!h->defer) {  // (deferred: the next iteration's move gathers the rows)
     SMC_RANGE("redistribute");
-    SMC_TRY(h, launch_redistribute(redist_args(h, 0), s));
+    SMC_TRY(h, launch_redistribute(iter_redist_args(h), s));
   }
   SMC_TRY(h, rec(6));
   {
-    SMC_RANGE("commit");
-    SMC_TRY(h, launch_commit(h->st, h->d, 0, 1, s, h->defer ? 1 : 0));
+    SMC_RANGE("commit");  // (part of the iteration's last kernel)
   }
   SMC_TRY(h, rec(7));
   return SMC_OK;

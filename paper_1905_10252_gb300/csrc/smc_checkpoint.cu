@@ -113,6 +113,11 @@ int smc_checkpoint_load(smc_sampler* h, const void* host_src, size_t bytes) {
   // first in use), whatever the saving sampler's were
   st.rs_dirty = 0;
   st.rs_w = 0;
+  // what lives only inside an iteration, at its value between iterations
+  // (a blob written before these fields existed holds padding there)
+  st.sub_ready = 0;
+  st.mkey = kNoMaxKey;
+  st.tickets = 0;
   st.trace = nullptr;
   st.mean_out = nullptr;
   st.fhat_out = nullptr;

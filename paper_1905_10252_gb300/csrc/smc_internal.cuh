@@ -42,6 +42,9 @@ constexpr uint32_t kPurposeInit = 1;
 constexpr uint32_t kPurposeMove = 2;
 constexpr uint32_t kPurposeResample = 3;
 
+// The ordered key (below) of -infinity: no maximum yet.
+constexpr long long kNoMaxKey = (long long)0x800FFFFFFFFFFFFFull;
+
 // ---------------------------------------------------------------- device state
 struct alignas(256) DevState {
   int64_t t;            // iteration index (0 after smc_init)
@@ -93,6 +96,12 @@ struct alignas(256) DevState {
   int32_t est_ready;    // 1: this iteration's move kernel wrote the eq. (7) tile records
   unsigned long long survivors;  // particles with ncopies > 0 in the current resampling
   smc_iter_stats last;  // statistics of the last finalised iteration
+  // smc_step's own iterations (FusedIter): the maximum of log w as an ordered
+  // key, raised by the move kernel's blocks and back at -inf between
+  // iterations, and the blocks of the iteration's last kernel that are done
+  long long mkey;
+  unsigned int tickets;
+  unsigned int tickets_pad;
 };
 
 // The run-start array in use: rs1 (the second array of a sampler that has
@@ -419,6 +428,34 @@ __device__ __forceinline__ long long warp_max_ll(long long v) {
   return v;
 }
 
+
+// ---------------------------------------------------------------- exact quotient
+// floor(n 2^64 / S) for 1 <= n < 2^31, n < S < 2^63: the reciprocal of S by
+// two Newton steps in 64-bit fixed point from the FP32 reciprocal (any seed
+// within 2^-18 will do), the quotient from it, and exact 128-bit corrections.
+// (The compiler's 128-bit division took about 4 us of one thread.)
+__device__ __forceinline__ uint64_t quotient_2p64(uint64_t n, uint64_t S) {
+  const int s = __clzll((long long)S);
+  const uint64_t Sn = S << s, u1 = n << s;  // n 2^64 / S = u1 / (Sn 2^-64)
+  const float d = float(uint32_t(Sn >> 40)) * 0x1p-24f;  // Sn 2^-64 in [1/2, 1), truncated
+  uint64_t V = uint64_t((1.0f / d) * 0x1p61f);  // ~2^61 / (Sn 2^-64), at most about 2^62
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const long long e = (long long)((1ull << 61) - __umul64hi(Sn, V));
+    V += uint64_t(__mul64hi((long long)V, e * 8));
+  }
+  uint64_t q = (__umul64hi(u1, V) << 3) | ((u1 * V) >> 61);
+  u128 rem = (u128(u1) << 64) - u128(q) * Sn;  // (mod 2^128: negative when q is too large)
+  while (rem >> 127) {
+    --q;
+    rem += Sn;
+  }
+  while (rem >= Sn) {
+    ++q;
+    rem -= Sn;
+  }
+  return q;
+}
 
 // ---------------------------------------------------------------- end of an iteration
 // Ends iteration t, executed by one full warp: swap buffers if resampled (or

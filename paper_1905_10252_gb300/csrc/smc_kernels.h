@@ -66,6 +66,7 @@ inline int lanes_per_particle(int, int) { return 1; }
 enum {
   PA_INIT_SKIP_LOGPI = 1,  // init writes log pi = 0 (a later likelihood pass adds it)
   PA_STALL_COPIES = 2,     // test hook: the tensor-core likelihood issues no data copies
+  PA_FUSED_ITER = 4,       // an iteration of smc_step: iteration st->t + 1, the maximum of log w into st->mkey
 };
 
 struct ParticleArgs {
@@ -121,6 +122,11 @@ struct QuantArgs {
   // kernel's tile records (epart) instead of reading x
   const double* epart;
   int32_t est_src;
+  // 1: a pass of smc_step's own iteration (launch_iter_*): the maximum comes
+  // from st->mkey, rows a gathering move has just written from the other
+  // buffer, and the iteration's bookkeeping is part of these kernels
+  int32_t fused;
+  int32_t defer;       // fused: a resampled iteration leaves its copy to the next move
   int32_t pad2;
 };
 
@@ -156,6 +162,7 @@ struct RedistArgs {
   DevState* st;
   int32_t stateful;      // 1: choose buffers by st->cur, honour st->flag / st->err
   int32_t use_pending;   // stateful: copy iff st->pending (a deferred resampling), not st->flag
+  int32_t end_iter;      // 1: the last block to finish ends the iteration (end_iteration)
   // stamped calls (see NcScanArgs::stamps): per tile, nonzero when the tile
   // has run starts (its runstart slice is then fully written; otherwise the
   // slice is not read and means -1 throughout); NULL: read every slice
@@ -244,6 +251,10 @@ bool quant_split(int64_t n);  // csub is used at this size
 cudaError_t launch_quant_reduce(const QuantArgs& a, cudaStream_t s);
 cudaError_t launch_quant_finalize(const QuantArgs& a, int set_lse_prev, cudaStream_t s);
 cudaError_t launch_quant_scan(const QuantArgs& a, cudaStream_t s);
+// smc_step's own iteration (QuantArgs::fused): the sums' finaliser, and the
+// scan with the iteration's statistics in one more block
+cudaError_t launch_iter_finalize(const QuantArgs& a, cudaStream_t s);
+cudaError_t launch_iter_scan(const QuantArgs& a, cudaStream_t s);
 cudaError_t launch_nc_reduce(const NcScanArgs& a, cudaStream_t s);
 cudaError_t launch_nc_finalize(const NcScanArgs& a, cudaStream_t s);
 cudaError_t launch_nc_scan(const NcScanArgs& a, cudaStream_t s);
