@@ -388,7 +388,7 @@ __device__ __forceinline__ void warp_write_est(float em, double R, float (&v)[DM
 // does not wait on memory:
 //   stage[0, 256)   rs[k0 .. k0 + 256)    (entries at or beyond n: masked)
 //   stage[256, 288) rs[k0 - 32 .. k0)     (the first step of the backward search)
-//   stage[288]      tile_src[k0 / 2048]
+//   stage[288]      tile_src[k0 / kRTile]
 // tile_sources_issue starts the copies; tile_sources_finish waits for them
 // and writes the tile's 256 sources to out[] (clamped into [0, n), as the copy
 // kernel clamps them).  Every lane of the warp takes part in both.

@@ -13,7 +13,7 @@
 //  * Redistribute (Algorithm 5 as the definition of the output): output-tile
 //    parallel gather.  The scan pass writes runstart[off_i] = i for every
 //    survivor (a run of ncopies_i output rows starts at off_i) and the source
-//    row of each tile's first output row; a tile of 2048 output rows loads its
+//    row of each tile's first output row; a tile of output rows loads its
 //    slice of runstart (resetting it to -1 for the next iteration), a block
 //    max-scan turns it into src(k), and the rows are copied with 16-byte
 //    vector loads/stores.  Every tile does the same bounded work whatever the
@@ -1092,8 +1092,9 @@ __device__ __forceinline__ void iter_stats(const QuantArgs& a, IterStatsSmem& sm
       mc = se_d > 0.0 ? sm.sxsum[tid] / se_d : st->mean[tid];
     }
     const double M = fmax(rmax, logc);
-    const double sc = (rmax == -INFINITY) ? 0.0 : exp(__dsub_rn(rmax, M));
-    const double e = exp(__dsub_rn(logc, M));
+    // (one of the two exponents is 0, and e^0 = 1)
+    const double sc = (rmax == -INFINITY) ? 0.0 : (rmax == M ? 1.0 : exp(__dsub_rn(rmax, M)));
+    const double e = logc == M ? 1.0 : exp(__dsub_rn(logc, M));
     const double den = __fma_rn(rden, sc, e);
     if (tid < a.d) {
       st->mean[tid] = mc;
@@ -1474,7 +1475,7 @@ __global__ void __launch_bounds__(kFinThreads) k_nc_finalize(NcScanArgs a) { nc_
 // run start (over all of itself if those overflow a queue), before its run
 // starts -- every slice the copy reads is then written in this call.
 constexpr int kNcWin = 8192;
-constexpr int kFillTiles = 128;
+constexpr int kFillTiles = 1024;
 constexpr uint64_t kFillAll = 1u << 17;
 
 __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
@@ -1573,13 +1574,16 @@ __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
 // ---------------------------------------------------------------- redistribute
 // Shared memory of one redistribute block, declared by the calling kernel so
 // that kernels dispatching to several row sizes hold one copy.
-struct RedistSmem {
-  int32_t mark[kRTile];
+template <int TILE>
+struct RedistSmemT {
+  int32_t mark[TILE];
   int32_t wsc[kRThreads / 32];
 };
+using RedistSmem = RedistSmemT<kCopyTile>;
 
-template <typename V, int CPR, int KU = 8, bool COH = false>
-__device__ __forceinline__ void redistribute_body(const RedistArgs& a, const int blk, RedistSmem& sm) {
+// One tile of TILE output rows, a whole number of kRTile.
+template <typename V, int CPR, int KU = 8, bool COH = false, int TILE = kCopyTile>
+__device__ __forceinline__ void redistribute_body(const RedistArgs& a, const int blk, RedistSmemT<TILE>& sm) {
   int cur = 0;
   if (a.stateful) {
     if (a.use_pending ? !a.st->pending : !(a.force || a.st->flag)) return;
@@ -1590,59 +1594,65 @@ __device__ __forceinline__ void redistribute_body(const RedistArgs& a, const int
   int32_t* const mark = sm.mark;
   int32_t* const wsc = sm.wsc;
   const int64_t n = a.n;
-  const int64_t k0 = int64_t(blk) * kRTile;
-  const int len = int(n - k0 < kRTile ? n - k0 : int64_t(kRTile));
+  const int64_t k0 = int64_t(blk) * TILE;
+  const int len = int(n - k0 < TILE ? n - k0 : int64_t(TILE));
   // this tile's slice of runstart (survivor runs starting here), reset to -1
   // for the next resampling
   int32_t* __restrict__ rs = rs_now(a.runstart, a.runstart_alt, a.st) + k0;
-  // (a stamped stateless call: an unstamped tile has no run starts, and its
-  // slice is neither read nor reset)
-  const bool read = !a.stamps || a.stamps[blk];
-  {
-    constexpr int kItems = kRTile / kRThreads;
-    int32_t v[kItems];
+  constexpr int kItems = TILE / kRThreads;
+  static_assert(TILE % kRTile == 0 && kRTile % kRThreads == 0, "whole rounds of the block per source entry");
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int32_t v[kItems];
 #pragma unroll
-    for (int u = 0; u < kItems; ++u) {
-      const int k = threadIdx.x + u * kRThreads;
-      v[u] = (read && k < len) ? rs[k] : -1;
-    }
-#pragma unroll
-    for (int u = 0; u < kItems; ++u) {
-      const int k = threadIdx.x + u * kRThreads;
-      // reset only the entries that were set (rewriting the whole slice was
-      // measured slower); stamped calls need no reset
-      if (!a.stamps && k < len && v[u] >= 0) rs[k] = -1;
-      mark[k] = v[u] < int32_t(n) ? v[u] : int32_t(n - 1);
-    }
+  for (int u = 0; u < kItems; ++u) {
+    const int k = threadIdx.x + u * kRThreads;
+    // (a stamped stateless call: an unstamped kRTile has no run starts, and
+    // its slice is neither read nor reset)
+    const bool read = !a.stamps || (k < len && a.stamps[blk * (TILE / kRTile) + u * kRThreads / kRTile]);
+    v[u] = (read && k < len) ? rs[k] : -1;
   }
-  __syncthreads();
-  if (failed) return;
   // the run covering the first output row may have started in an earlier tile
-  if (threadIdx.x == 0) {
-    const int32_t first = min(max(a.tile_src[blk], 0), int32_t(n - 1));
-    mark[0] = max(mark[0], first);
+  const int32_t first =
+      threadIdx.x == 0 ? min(max(a.tile_src[int64_t(blk) * (TILE / kRTile)], 0), int32_t(n - 1)) : -1;
+#pragma unroll
+  for (int u = 0; u < kItems; ++u) {
+    const int k = threadIdx.x + u * kRThreads;
+    // reset only the entries that were set (rewriting the whole slice was
+    // measured slower); stamped calls need no reset
+    if (!a.stamps && k < len && v[u] >= 0) rs[k] = -1;
+    v[u] = v[u] < int32_t(n) ? v[u] : int32_t(n - 1);
   }
-  __syncthreads();
-  // inclusive max-scan of mark[0, kRTile): 16 consecutive entries per thread
-  {
-    constexpr int kItems = kRTile / kRThreads;
-    const int b = threadIdx.x * kItems;
-    int run = -1;
+  v[0] = max(v[0], first);
+  if (failed) return;
+  // inclusive max-scan over the tile: kItems consecutive entries per thread
+  // (one: straight from the register)
+  int run = v[0];
+  const int b = threadIdx.x * kItems;
+  if constexpr (kItems > 1) {
+#pragma unroll
+    for (int u = 0; u < kItems; ++u) mark[threadIdx.x + u * kRThreads] = v[u];
+    __syncthreads();
+    run = -1;
 #pragma unroll
     for (int q = 0; q < kItems; ++q) run = max(run, mark[b + q]);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int incl = warp_incl_max_i32(run);
+  }
+  {
+    const int incl = warp_incl_max_i32(run);
     if (lane == 31) wsc[wid] = incl;
     __syncthreads();
     int carry = -1;
     for (int w = 0; w < wid; ++w) carry = max(carry, wsc[w]);
-    int excl = __shfl_up_sync(0xffffffffu, incl, 1);
-    if (lane == 0) excl = -1;
-    run = max(carry, excl);
+    if constexpr (kItems > 1) {
+      int excl = __shfl_up_sync(0xffffffffu, incl, 1);
+      if (lane == 0) excl = -1;
+      run = max(carry, excl);
 #pragma unroll
-    for (int q = 0; q < kItems; ++q) {
-      run = max(run, mark[b + q]);
-      mark[b + q] = run;
+      for (int q = 0; q < kItems; ++q) {
+        run = max(run, mark[b + q]);
+        mark[b + q] = run;
+      }
+    } else {
+      mark[threadIdx.x] = max(carry, incl);
     }
   }
   __syncthreads();
@@ -1684,26 +1694,26 @@ __device__ __forceinline__ void redistribute_body(const RedistArgs& a, const int
   }
 }
 
-template <typename V, int CPR>
+template <typename V, int CPR, int TILE>
 __global__ void __launch_bounds__(kRThreads) k_redistribute(RedistArgs a) {
-  __shared__ RedistSmem sm;
-  redistribute_body<V, CPR>(a, blockIdx.x, sm);
+  __shared__ RedistSmemT<TILE> sm;
+  redistribute_body<V, CPR, 8, false, TILE>(a, blockIdx.x, sm);
   if (a.end_iter) end_iteration(a.st, gridDim.x, 0);
 }
 
 // ---------------------------------------------------------------- one-tile samplers
-// A sampler whose N fits one copy tile (N <= 2048) runs redistribute and
-// commit as one kernel.
+// A fused small sampler (N <= kSmallTile) that also returns the covariance
+// ends its last iteration with redistribute and commit as one kernel.
 template <typename V, int CPR>
 __global__ void __launch_bounds__(kRThreads) k_redistribute_commit(RedistArgs a, int d, int force_flip, int recycle) {
-  __shared__ RedistSmem sm;
-  redistribute_body<V, CPR>(a, 0, sm);
+  __shared__ RedistSmemT<kSmallTile> sm;
+  redistribute_body<V, CPR, 8, false, kSmallTile>(a, 0, sm);
   __syncthreads();
   if (threadIdx.x < 32) commit_warp(a.st, d, force_flip, recycle);
 }
 
 // ---------------------------------------------------------------- fused small-sampler iterations
-// FP64 samplers of one quantise block and one copy tile (N <= 2048): k
+// FP64 samplers of one quantise block and kSmallTile rows (N <= 2048): k
 // iterations of Algorithm 2 in one cooperative launch.  Every block runs its
 // share of the move + reweight with the particle-to-thread map of the
 // separate move launch (move_threads per block own particles); then block 0
@@ -1773,7 +1783,7 @@ union SmallIterSmem {
   TargetSmem<double> ts;
   QuantReduceSmem q;
   ScanSmem sc;
-  RedistSmem r;
+  RedistSmemT<kSmallTile> r;
 };
 
 template <int DMAX, typename V>
@@ -1781,7 +1791,7 @@ __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
   __shared__ SmallIterSmem sm;
   TargetSmem<double>& ts = sm.ts;
   QuantReduceSmem& qsm = sm.q;
-  RedistSmem& rsm = sm.r;
+  RedistSmemT<kSmallTile>& rsm = sm.r;
   DevState* st = s.a.st;
   unsigned long long* const bar = s.bar;
   unsigned long long nbar = 0;
@@ -1804,7 +1814,7 @@ __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
         quant_scan_body<8>(s.q, 0, s.q.cbase[0], sm.sc);
       if (!(s.stop_last && it + 1 == s.k)) {
         __syncthreads();
-        redistribute_body<V, 0, 8, true>(s.r, 0, rsm);
+        redistribute_body<V, 0, 8, true, kSmallTile>(s.r, 0, rsm);
         __syncthreads();
         if (threadIdx.x < 32) commit_warp(st, s.d, 0, 1);
       }
@@ -1813,7 +1823,7 @@ __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
   }
 }
 
-bool small_iter_fits(int64_t n, int dtype) { return dtype == SMC_F64 && n <= kRTile && n <= kQTile; }
+bool small_iter_fits(int64_t n, int dtype) { return dtype == SMC_F64 && n <= kSmallTile && n <= kQTile; }
 
 template <int DMAX>
 static cudaError_t iterate_small_d(const SmallIterArgs& s, int blocks, cudaStream_t st) {
@@ -1909,11 +1919,13 @@ __global__ void __launch_bounds__(kRThreads) k_identity_runs_batch(const RedistA
                                                                   const int4* __restrict__ map) {
   const int4 m = map[blockIdx.x];
   const RedistArgs a = ra[m.x];
-  const int64_t k0 = int64_t(m.y) * kRTile;
-  const int len = int(a.n - k0 < kRTile ? a.n - k0 : int64_t(kRTile));
+  const int64_t k0 = int64_t(m.y) * kCopyTile;
+  const int len = int(a.n - k0 < kCopyTile ? a.n - k0 : int64_t(kCopyTile));
   int32_t* __restrict__ rs = rs_now(a.runstart, a.runstart_alt, a.st);
-  for (int k = threadIdx.x; k < len; k += kRThreads) rs[k0 + k] = int32_t(k0 + k);
-  if (threadIdx.x == 0) const_cast<int32_t*>(a.tile_src)[m.y] = int32_t(k0);
+  for (int k = threadIdx.x; k < len; k += kRThreads) {
+    rs[k0 + k] = int32_t(k0 + k);
+    if (k % kRTile == 0) const_cast<int32_t*>(a.tile_src)[(k0 + k) / kRTile] = int32_t(k0 + k);
+  }
 }
 
 cudaError_t launch_quant_reduce_batch(const QuantArgs* qa, const int4* map, int nblocks, cudaStream_t s,
@@ -2040,33 +2052,50 @@ cudaError_t launch_nc_scan(const NcScanArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_redistribute(const RedistArgs& a, cudaStream_t s) {
-  const int grid = int((a.n + kRTile - 1) / kRTile);
+constexpr int64_t kSmallCopy = 2 << 20;
+
+template <int TILE>
+static void redistribute_t(const RedistArgs& a, cudaStream_t s) {
+  const int grid = int((a.n + TILE - 1) / TILE);
   const int rb = a.row_bytes;
   if (rb % 16 == 0) {
     switch (rb / 16) {
-      case 1: k_redistribute<uint4, 1><<<grid, kRThreads, 0, s>>>(a); break;
-      case 2: k_redistribute<uint4, 2><<<grid, kRThreads, 0, s>>>(a); break;
-      case 4: k_redistribute<uint4, 4><<<grid, kRThreads, 0, s>>>(a); break;
-      case 8: k_redistribute<uint4, 8><<<grid, kRThreads, 0, s>>>(a); break;
-      default: k_redistribute<uint4, 0><<<grid, kRThreads, 0, s>>>(a); break;
+      case 1: k_redistribute<uint4, 1, TILE><<<grid, kRThreads, 0, s>>>(a); break;
+      case 2: k_redistribute<uint4, 2, TILE><<<grid, kRThreads, 0, s>>>(a); break;
+      case 4: k_redistribute<uint4, 4, TILE><<<grid, kRThreads, 0, s>>>(a); break;
+      case 8: k_redistribute<uint4, 8, TILE><<<grid, kRThreads, 0, s>>>(a); break;
+      default: k_redistribute<uint4, 0, TILE><<<grid, kRThreads, 0, s>>>(a); break;
     }
   } else if (rb % 8 == 0) {
     if (rb == 8)
-      k_redistribute<uint2, 1><<<grid, kRThreads, 0, s>>>(a);
+      k_redistribute<uint2, 1, TILE><<<grid, kRThreads, 0, s>>>(a);
     else
-      k_redistribute<uint2, 0><<<grid, kRThreads, 0, s>>>(a);
+      k_redistribute<uint2, 0, TILE><<<grid, kRThreads, 0, s>>>(a);
   } else {
     if (rb == 4)
-      k_redistribute<uint32_t, 1><<<grid, kRThreads, 0, s>>>(a);
+      k_redistribute<uint32_t, 1, TILE><<<grid, kRThreads, 0, s>>>(a);
     else
-      k_redistribute<uint32_t, 0><<<grid, kRThreads, 0, s>>>(a);
+      k_redistribute<uint32_t, 0, TILE><<<grid, kRThreads, 0, s>>>(a);
   }
+}
+
+cudaError_t launch_redistribute(const RedistArgs& a, cudaStream_t s) {
+  // Up to kSmallCopy rows a block copies kRTile = 512 of them, above kCopyTile =
+  // 1024.  A block's time is mostly latency (its run starts, the scan, the
+  // gather), so a small copy needs many: 10 blocks of 2048 rows took 17.5 us
+  // of an iteration at N = 20011, D = 32 (iteration 47.8 -> 41.6 us); a large one
+  // fills the SMs either way and moves more bytes per block with 1024
+  // (iteration at N = 2^24, D = 16 1.030 ms, with 512 1.046; at N = 2^20, D = 32
+  // 0.171 and 0.169).
+  if (a.n <= kSmallCopy)
+    redistribute_t<kRTile>(a, s);
+  else
+    redistribute_t<kCopyTile>(a, s);
   return cudaGetLastError();
 }
 
 cudaError_t launch_redistribute_commit(const RedistArgs& a, int d, int force_flip, int recycle, cudaStream_t s) {
-  if (a.n > kRTile) return cudaErrorInvalidValue;
+  if (a.n > kSmallTile) return cudaErrorInvalidValue;
   const int rb = a.row_bytes;
   if (rb % 16 == 0) {
     switch (rb / 16) {

@@ -231,7 +231,7 @@ RedistArgs redist_args(const smc_sampler* h, int force) {
   r.runstart = h->rs;
   r.runstart_alt = h->rs_alt;
   r.tile_src = h->tile_src;
-  r.ntiles = h->L.ntiles;
+  r.ntiles = int32_t(div_up(h->n, kCopyTile));
   r.force = force;
   r.x_in[0] = h->x[0];
   r.x_in[1] = h->x[1];
@@ -482,11 +482,10 @@ int smc_init(smc_sampler** out, const smc_config* cfg, void* x_dev, void* x_alt_
   h->gp_ready = false;
   // deferred redistribution: the gathering move is the records kernel's, and
   // the quantise and copy passes span several blocks
-  h->defer = (cfg->flags & SMC_FLAG_DEFER_REDISTRIBUTE) && est_in_move(h) && h->L.qblocks > 1 && h->L.ntiles > 1;
-  // small FP64 samplers (generic move kernel, one quantise block, one copy
-  // tile): smc_step fuses their iterations into one cooperative launch
-  h->small_iter = small_iter_fits(h->n, h->dtype) && cfg->target != SMC_LOGISTIC && !h->defer &&
-                  h->L.qblocks == 1 && h->L.ntiles == 1;
+  h->defer = (cfg->flags & SMC_FLAG_DEFER_REDISTRIBUTE) && est_in_move(h) && h->L.qblocks > 1;
+  // small FP64 samplers (generic move kernel, one quantise block, one block's
+  // copy): smc_step fuses their iterations into one cooperative launch
+  h->small_iter = small_iter_fits(h->n, h->dtype) && cfg->target != SMC_LOGISTIC && !h->defer && h->L.qblocks == 1;
   if (e != cudaSuccess) {
     int r = cuda_fail(nullptr, e, "smc_init launch");
     delete h;
@@ -778,7 +777,7 @@ int redistribute_raw_impl(int64_t n, int32_t row_bytes, const int32_t* ncopies_d
   r.lp_bytes = 0;
   r.runstart = a.runstart;
   r.tile_src = a.tile_src;
-  r.ntiles = L.ntiles;
+  r.ntiles = int32_t(div_up(n, kCopyTile));
   r.force = 1;
   r.x_in[0] = r.x_in[1] = in_dev;
   r.x_out[0] = r.x_out[1] = out_dev;

@@ -59,7 +59,7 @@ Plan make_plan(smc_sampler* const* m, int count, int sms) {
   for (int s : order) {
     const int nq = int(div_up(m[s]->n, kQTile));
     for (int j = 0; j < nq; ++j) p.qmap.push_back(make_int4(s, j, nq, 0));
-    const int nr = int(div_up(m[s]->n, kRTile));
+    const int nr = int(div_up(m[s]->n, kCopyTile));
     for (int j = 0; j < nr; ++j) p.rmap.push_back(make_int4(s, j, nr, 0));
   }
   for (int v = 0; v < SMC_BATCH_MOVE_VARIANTS; ++v) {

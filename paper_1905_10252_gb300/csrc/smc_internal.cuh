@@ -29,7 +29,9 @@ constexpr int kQThreads = 256;        // 16 consecutive elements per thread
 constexpr int kQItems = kQTile / kQThreads;
 constexpr int kQSplit = 8;            // blocks that share a tile in the passes of small samplers
 constexpr int kQSplitTiles = 76;       // ... of at most this many tiles
-constexpr int kRTile = 2048;          // output rows per block of the redistribute copy
+constexpr int kRTile = 512;            // output rows per source entry (tile_src, stamps) of the redistribute copy
+constexpr int kCopyTile = 1024;        // output rows per block of the copy of large samplers and of batches
+constexpr int kSmallTile = 2048;      // ... of the one-block copy of a fused small sampler
 constexpr int kRThreads = 256;
 constexpr int kPThreads = 256;        // particle kernels (init / move / reweight)
 constexpr int kFinThreads = 1024;     // single-block finalisers

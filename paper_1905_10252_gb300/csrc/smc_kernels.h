@@ -151,7 +151,7 @@ struct RedistArgs {
   int32_t* runstart;     // consumed and reset to -1 by the tile that reads it
   int32_t* runstart_alt; // second run-start array (NULL: one array); st->rs_w picks
   const int32_t* tile_src;
-  int32_t ntiles;
+  int32_t ntiles;        // copy tiles (kCopyTile rows) of a batched launch
   int32_t force;         // copy even if the decision is "no resample"
   const void* x_in[2];   // indexed by the current buffer (stateful) or [0]
   void* x_out[2];
@@ -259,7 +259,7 @@ cudaError_t launch_nc_reduce(const NcScanArgs& a, cudaStream_t s);
 cudaError_t launch_nc_finalize(const NcScanArgs& a, cudaStream_t s);
 cudaError_t launch_nc_scan(const NcScanArgs& a, cudaStream_t s);
 cudaError_t launch_redistribute(const RedistArgs& a, cudaStream_t s);
-// one-tile samplers (N <= 2048): redistribute + commit as one launch
+// fused small samplers (N <= kSmallTile): redistribute + commit as one launch
 cudaError_t launch_redistribute_commit(const RedistArgs& a, int d, int force_flip, int recycle, cudaStream_t s);
 
 // k iterations of an FP64 sampler of one quantise block and one copy tile

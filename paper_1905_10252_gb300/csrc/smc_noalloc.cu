@@ -115,7 +115,7 @@ extern "C" int smc_redistribute_raw_noalloc(int64_t n, int32_t row_bytes, const 
   r.lp_bytes = 0;
   r.runstart = a.runstart;
   r.tile_src = a.tile_src;
-  r.ntiles = a.ntiles;
+  r.ntiles = int32_t((n + kCopyTile - 1) / kCopyTile);
   r.force = 1;
   r.x_in[0] = r.x_in[1] = in_dev;
   r.x_out[0] = r.x_out[1] = out_dev;

@@ -66,7 +66,7 @@ SlotsPlan make_slots_plan(const int64_t* cap, int count, int sms) {
     p.nb[s] = std::max(1, std::min(b, full));
   }
   for (int s : order) {
-    const int nq = int(div_up(cap[s], kQTile)), nr = int(div_up(cap[s], kRTile));
+    const int nq = int(div_up(cap[s], kQTile)), nr = int(div_up(cap[s], kCopyTile));
     for (int j = 0; j < nq; ++j) p.qmap.push_back(make_int4(s, j, nq, 0));
     for (int j = 0; j < nr; ++j) p.rmap.push_back(make_int4(s, j, nr, 0));
     for (int j = 0; j < p.nb[s]; ++j) p.mmap.push_back(make_int4(s, j, p.nb[s], 0));
@@ -297,7 +297,7 @@ cudaError_t write_compact_maps(smc_slots* b) {
   for (int s : order) {
     const smc_sampler* h = b->m[s];
     if (!h) continue;
-    const int hq = h->L.qblocks, hr = h->L.ntiles, hm = b->plan.nb[s];
+    const int hq = h->L.qblocks, hr = int(div_up(h->n, kCopyTile)), hm = b->plan.nb[s];
     for (int j = 0; j < hq; ++j) q[nq++] = make_int4(s, j, hq, 0);
     for (int j = 0; j < hr; ++j) r[nr++] = make_int4(s, j, hr, 0);
     for (int j = 0; j < hm; ++j) m[nm++] = make_int4(s, j, hm, 0);
