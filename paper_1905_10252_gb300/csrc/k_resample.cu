@@ -139,40 +139,30 @@ __global__ void k_state_init(DevState* st, int64_t n, int64_t t, int F) {
 }
 
 // ---------------------------------------------------------------- max of log w (stateless path)
-// part[b] = {max, number of finite entries}; NaN is an error.
-__global__ void __launch_bounds__(kQThreads) k_max_logw(const double* __restrict__ logw, int64_t n,
-                                                       double* __restrict__ part, DevState* st) {
-  __shared__ double shm[kQThreads / 32], shc[kQThreads / 32];
-  double m = -INFINITY, cnt = 0.0;
-  bool nan = false;
-  const int64_t base = int64_t(blockIdx.x) * kQTile;
-#pragma unroll 4
+// Raises st->mkey; NaN is an error.  Integer-ordered keys with every load of a
+// thread in flight: FP64 comparisons and a count (two lanes per SM and clock
+// each) took 155 us at N = 2^24, 27 now.
+__global__ void __launch_bounds__(kQThreads) k_max_logw(const double* __restrict__ logw, int64_t n, DevState* st) {
+  __shared__ long long shm[kQThreads / 32];
+  MaxTracker mt;
+  mt.init();
+  const int64_t base = int64_t(blockIdx.x) * kQTile + threadIdx.x;
+  double v[kQItems];
+#pragma unroll
   for (int k = 0; k < kQItems; ++k) {
-    const int64_t i = base + k * kQThreads + threadIdx.x;
-    if (i < n) {
-      const double v = logw[i];
-      nan |= isnan(v);
-      if (v > -INFINITY) cnt += 1.0;
-      m = fmax(m, v);
-    }
+    const int64_t i = base + k * kQThreads;
+    v[k] = i < n ? __ldg(logw + i) : -INFINITY;
   }
-  if (nan) record_error(st, SMC_ENONFINITE);
-  m = warp_max(m);
-  cnt = warp_sum(cnt);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    shm[wid] = m;
-    shc[wid] = cnt;
-  }
+#pragma unroll
+  for (int k = 0; k < kQItems; ++k) mt.add(v[k]);
+  if (mt.nan) record_error(st, SMC_ENONFINITE);
+  const long long wm = warp_max_ll(mt.best);
+  if ((threadIdx.x & 31) == 0) shm[threadIdx.x >> 5] = wm;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double mm = -INFINITY, cc = 0.0;
-    for (int w = 0; w < kQThreads / 32; ++w) {
-      mm = fmax(mm, shm[w]);
-      cc += shc[w];
-    }
-    part[2 * blockIdx.x] = mm;
-    part[2 * blockIdx.x + 1] = cc;
+    long long m = shm[0];
+    for (int w = 1; w < kQThreads / 32; ++w) m = shm[w] > m ? shm[w] : m;
+    if (m > *const_cast<volatile long long*>(&st->mkey)) atomicMax(&st->mkey, m);
   }
 }
 
@@ -1129,6 +1119,17 @@ __device__ __forceinline__ void iter_stats(const QuantArgs& a, IterStatsSmem& sm
     recs[k]->resampled = flag;
     recs[k]->t = t;
   }
+  if (a.stats_out) {
+    smc_iter_stats r;
+    r.lse = lse;
+    r.logc = logc;
+    r.ess = sm.ess;
+    r.max_logw = m;
+    r.resampled = flag;
+    r.t = t;
+    r.survivors = 0;
+    *a.stats_out = r;
+  }
 }
 
 // The end of an iteration, by the last block of its last kernel to finish (so
@@ -1199,9 +1200,8 @@ __device__ __forceinline__ void tile_starts_flush(int32_t* __restrict__ tile_src
 // Shared memory of the scan: the block's W staged for a blocked layout (then
 // its copy counts), the block scan's scratch and the long-run queue.
 struct ScanSmem {
-  union {
+  struct {
     uint64_t w[kQThreads * 17];
-    uint32_t o[kQThreads * 17];
   } buf;
   uint64_t scratch[33];
   BigRuns big;
@@ -1231,19 +1231,14 @@ __device__ __forceinline__ void quant_scan_body(const QuantArgs& a, const int64_
   }
   __syncthreads();
   const uint64_t S = st->S, U = st->U;
-  uint64_t W[ITEMS];
+  uint64_t* const mine = buf.w + threadIdx.x * (ITEMS + 1);
   uint64_t tsum = 0;
 #pragma unroll
-  for (int q = 0; q < ITEMS; ++q) {
-    W[q] = buf.w[threadIdx.x * (ITEMS + 1) + q];
-    tsum += W[q];
-  }
+  for (int q = 0; q < ITEMS; ++q) tsum += mine[q];
   uint64_t btot;
-  uint64_t C = C0 + block_excl_scan_u64(tsum, scratch, &btot);
-  uint32_t ncv[ITEMS];
+  const uint64_t C = C0 + block_excl_scan_u64(tsum, scratch, &btot);
   unsigned nsurv = 0;
-  // off_i = floor((N C_{i-1} + U) / S) for every item independently (no
-  // serial dependency between items): the estimate mulhi(C, floor(N 2^64/S))
+  // off_i = floor((N C_{i-1} + U) / S): the estimate mulhi(C, floor(N 2^64/S))
   // is at most 2 below floor(N C / S), and floor((N C + U)/S) is at most 1
   // above that; exact 128-bit comparisons fix the result.
   const uint64_t Rn = st->recip;  // floor(N 2^64 / S)
@@ -1262,70 +1257,39 @@ __device__ __forceinline__ void quant_scan_body(const QuantArgs& a, const int64_
       }
     return qq;
   };
-  if (!a.ncopies) {
-    // no copy counts to return (the sampler's own resampling): the items
-    // one after another, each offset computed as it is needed -- the same
-    // integers as below, from a short loop instead of ITEMS + 1 unrolled
-    // quotients (which overflowed the instruction cache)
-    const int64_t i0 = base + int64_t(threadIdx.x) * ITEMS;
-    uint64_t cp = C, op = quot(C);
+  // the items one after another, each offset computed as it is needed, from a
+  // short loop (ITEMS + 1 unrolled quotients overflow the instruction cache:
+  // 125 instead of 96 us at N = 2^24 with copy counts)
+  const int64_t i0 = base + int64_t(threadIdx.x) * ITEMS;
+  const bool counts = a.ncopies != nullptr;
+  uint64_t cp = C, op = quot(C);
 #pragma unroll 4
-    for (int q = 0; q < ITEMS; ++q) {
-      const uint64_t cn = cp + buf.w[threadIdx.x * (ITEMS + 1) + q];
-      const uint64_t on = quot(cn);
-      const int64_t i = i0 + q;
-      if (on > op && i < n) {
-        ++nsurv;
-        if (a.write_rs) rsa[op] = int32_t(i);
+  for (int q = 0; q < ITEMS; ++q) {
+    const uint64_t cn = cp + mine[q];
+    const uint64_t on = quot(cn);
+    const int64_t i = i0 + q;
+    if (counts) mine[q] = on - op;  // (the item's own W is done with)
+    if (on > op && i < n) {
+      ++nsurv;
+      if (a.write_rs) {  // (copy counts alone need no run starts or tile sources)
+        rsa[op] = int32_t(i);
         tile_starts_of_run(a.tile_src, op, on, uint64_t(n), int32_t(i), big);
       }
-      cp = cn;
-      op = on;
     }
-    tile_starts_flush(a.tile_src, big);
-    unsigned v = nsurv;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&const_cast<DevState*>(st)->survivors, (unsigned long long)v);
-    return;
+    cp = cn;
+    op = on;
   }
-  uint64_t Cx[ITEMS + 1];
-  Cx[0] = C;
+  tile_starts_flush(a.tile_src, big);  // (block barrier inside)
+  unsigned v = nsurv;
 #pragma unroll
-  for (int q = 0; q < ITEMS; ++q) Cx[q + 1] = Cx[q] + W[q];
-  uint64_t offs[ITEMS + 1];
-#pragma unroll
-  for (int q = 0; q <= ITEMS; ++q) offs[q] = quot(Cx[q]);
-  const int64_t i0 = base + int64_t(threadIdx.x) * ITEMS;
-#pragma unroll
-  for (int q = 0; q < ITEMS; ++q) {
-    const uint64_t lo = offs[q], hi = offs[q + 1];
-    ncv[q] = uint32_t(hi - lo);
-    const int64_t i = i0 + q;
-    if (hi > lo && i < n) {
-      ++nsurv;
-      if (a.write_rs) rsa[lo] = int32_t(i);
-      // every redistribute tile whose first output row lies in [lo, hi)
-      tile_starts_of_run(a.tile_src, lo, hi, uint64_t(n), int32_t(i), big);
-    }
-  }
-  tile_starts_flush(a.tile_src, big);
-  {
-    unsigned v = nsurv;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(&const_cast<DevState*>(st)->survivors, (unsigned long long)v);
-  }
-  __syncthreads();  // buf.w no longer read
-  if (a.ncopies) {
-#pragma unroll
-    for (int q = 0; q < ITEMS; ++q) buf.o[threadIdx.x * (ITEMS + 1) + q] = ncv[q];
-    __syncthreads();
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0 && v) atomicAdd(&const_cast<DevState*>(st)->survivors, (unsigned long long)v);
+  if (counts) {
 #pragma unroll 4
     for (int k = 0; k < ITEMS; ++k) {
       const int idx = k * kQThreads + threadIdx.x;
       const int64_t i = base + idx;
-      if (i < n) a.ncopies[i] = int32_t(buf.o[(idx / ITEMS) * (ITEMS + 1) + idx % ITEMS]);
+      if (i < n) a.ncopies[i] = int32_t(buf.w[(idx / ITEMS) * (ITEMS + 1) + idx % ITEMS]);
     }
   }
 }
@@ -1370,7 +1334,7 @@ __global__ void __launch_bounds__(kQThreads, 4) k_iter_scan(QuantArgs a) {
   } else if constexpr (SUB) {
     constexpr int kSub = kQTile / kQSplit;
     const int64_t base = int64_t(blk) * kSub;
-    if (base < a.n && !a.st->err && a.st->flag)
+    if (base < a.n && !a.st->err && (a.force || a.st->flag))
       quant_scan_body<kSub / kQThreads>(a, base, a.cbase[blk / kQSplit] + a.csub[blk], sm.scan);
   } else {
     quant_scan_body(a, int64_t(blk) * kQTile, a.cbase[blk], sm.scan);
@@ -1965,8 +1929,8 @@ cudaError_t launch_state_init(DevState* st, int64_t n, int64_t t, int F, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_max_logw(const double* logw, int64_t n, double* part, int nb, DevState* st, cudaStream_t s) {
-  k_max_logw<<<nb, kQThreads, 0, s>>>(logw, n, part, st);
+cudaError_t launch_max_logw(const double* logw, int64_t n, DevState* st, cudaStream_t s) {
+  k_max_logw<<<qblocks(n), kQThreads, 0, s>>>(logw, n, st);
   return cudaGetLastError();
 }
 

@@ -826,7 +826,6 @@ int smc_resample_raw(int64_t n, const double* logw_dev, uint64_t seed, uint64_t 
   char* ws = static_cast<char*>(ws_dev);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   DevState* st = reinterpret_cast<DevState*>(ws + L.st);
-  double* part = reinterpret_cast<double*>(ws + L.part);
   QuantArgs q{};
   q.n = n;
   q.logw = logw_dev;
@@ -845,12 +844,13 @@ int smc_resample_raw(int64_t n, const double* logw_dev, uint64_t seed, uint64_t 
   q.ntiles = L.ntiles;
   q.st = st;
   q.stats_out = stats_dev;
-  e = launch_state_init(st, n, int64_t(t), quant_shift(n), s);
-  if (e == cudaSuccess) e = launch_max_logw(logw_dev, n, part, L.qblocks, st, s);
-  if (e == cudaSuccess) e = launch_max_finalize(part, L.qblocks, st, s);
+  // the passes of smc_step's own iteration, from t - 1 to t
+  q.fused = 1;
+  e = launch_state_init(st, n, int64_t(t - 1), quant_shift(n), s);
+  if (e == cudaSuccess) e = launch_max_logw(logw_dev, n, st, s);
   if (e == cudaSuccess) e = launch_quant_reduce(q, s);
-  if (e == cudaSuccess) e = launch_quant_finalize(q, 0, s);
-  if (e == cudaSuccess) e = launch_quant_scan(q, s);
+  if (e == cudaSuccess) e = launch_iter_finalize(q, s);
+  if (e == cudaSuccess) e = launch_iter_scan(q, s);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "smc_resample_raw");
   return SMC_OK;
 }

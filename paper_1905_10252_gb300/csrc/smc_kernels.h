@@ -246,7 +246,7 @@ cudaError_t launch_take_errors_batch(const ParticleArgs* pa, int32_t* errs, int 
 // k_resample.cu
 cudaError_t upload_expfx_table();  // once per device, outside stream capture
 cudaError_t expfx_table(const uint64_t** out);  // its device address (after the upload)
-cudaError_t launch_max_logw(const double* logw, int64_t n, double* part, int nb, DevState* st, cudaStream_t s);
+cudaError_t launch_max_logw(const double* logw, int64_t n, DevState* st, cudaStream_t s);
 bool quant_split(int64_t n);  // csub is used at this size
 cudaError_t launch_quant_reduce(const QuantArgs& a, cudaStream_t s);
 cudaError_t launch_quant_finalize(const QuantArgs& a, int set_lse_prev, cudaStream_t s);
