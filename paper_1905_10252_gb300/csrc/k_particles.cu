@@ -25,46 +25,112 @@
 namespace smc {
 
 // ---------------------------------------------------------------- target set-up
-// One thread: Cholesky-Banachiewicz of Sigma (row by row, fma accumulation),
-// then P = L^-1 by forward substitution on the identity, and FP32 copies.
-__global__ void k_target_setup(TargetDev* tg, int kind, double nu, const double* __restrict__ mu,
-                               const double* __restrict__ sigma, int d, DevState* st) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  tg->kind = kind;
-  tg->d = d;
-  tg->nu = nu;
-  for (int c = 0; c < d; ++c) {
-    tg->mu[c] = mu[c];
-    tg->muf[c] = float(mu[c]);
+// Four warps: Cholesky of Sigma, then P = L^-1 by forward substitution on the
+// identity, and FP32 copies.  Lane i owns row i of L (then column i of P);
+// warp w keeps the unfinished sums of columns (rows of P) w, w + 4, ... in its
+// registers: once column k is done every later sum takes its term k, so that
+// each element adds its terms in the order k = 0, 1, ... of the row-by-row
+// form (fma accumulation), with many chains in flight instead of one.  A
+// warp's FP64 instruction takes 64 cycles of its quarter of the SM, hence the
+// four; and the sums move down one register every four steps, so that the
+// steps are a short loop body (written out for 32 columns, the instruction fetch
+// alone took 0.1 ms).  One thread walking all of it through global memory
+// took 1.01 ms at D = 32, 0.29 at D = 16, 0.115 at D = 4; 82, 37 and 10 us now.
+constexpr int kSetupWarps = 4;
+template <int DMAX>
+__global__ void __launch_bounds__(32 * kSetupWarps) k_target_setup(TargetDev* tg, int kind, double nu,
+                                                                 const double* __restrict__ mu,
+                                                                 const double* __restrict__ sigma, int d,
+                                                                 DevState* st) {
+  constexpr int kW = kSetupWarps, kJ = DMAX / kW;
+  __shared__ double sL[2 * DMAX][DMAX + 1];  // (rows DMAX .. are read past the last column: zero)
+  __shared__ double sp[32];
+  __shared__ int s_bad;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    tg->kind = kind;
+    tg->d = d;
+    tg->nu = nu;
+    s_bad = 0;
   }
-  if (tg->kind == SMC_STUDENT_T) return;
-  double* L = tg->L;
-  for (int i = 0; i < d * kMaxD; ++i) L[i] = 0.0;
-  for (int i = 0; i < d; ++i) {
-    for (int j = 0; j <= i; ++j) {
-      double s = 0.0;
-      for (int k = 0; k < j; ++k) s = __fma_rn(L[i * kMaxD + k], L[j * kMaxD + k], s);
-      if (i == j) {
-        const double dd = __dsub_rn(sigma[i * d + i], s);
-        if (!(dd > 0.0)) {
-          record_error(st, SMC_EINVAL);
+  if (threadIdx.x < d) {
+    tg->mu[lane] = mu[lane];
+    tg->muf[lane] = float(mu[lane]);
+  }
+  if (kind == SMC_STUDENT_T) return;
+  for (int e = threadIdx.x; e < 2 * DMAX * (DMAX + 1); e += blockDim.x) (&sL[0][0])[e] = 0.0;
+  // acc[j], row[j]: column base + 4 j + w
+  double acc[kJ + 1], row[kJ + 1];
+#pragma unroll
+  for (int j = 0; j <= kJ; ++j) {
+    const int c = kW * j + w;
+    acc[j] = 0.0;
+    row[j] = (lane < d && c < d) ? sigma[lane * d + c] : 0.0;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int base = 0; base < d; base += kW) {
+#pragma unroll
+    for (int o = 0; o < kW; ++o) {
+      const int k = base + o;
+      if (k < d) {
+        if (w == o) {
+          const double v = __dsub_rn(row[0], acc[0]);
+          double diag = 0.0;
+          if (lane == k) diag = v > 0.0 ? __dsqrt_rn(v) : -1.0;
+          diag = __shfl_sync(0xffffffffu, diag, k);
+          if (!(diag > 0.0)) s_bad = 1;  // not positive definite
+          if (lane < DMAX) sL[lane][k] = lane == k ? diag : (lane > k ? __ddiv_rn(v, diag) : 0.0);
+        }
+        __syncthreads();
+        if (s_bad) {
+          if (threadIdx.x == 0) record_error(st, SMC_EINVAL);
           return;
         }
-        L[i * kMaxD + i] = __dsqrt_rn(dd);
-      } else {
-        L[i * kMaxD + j] = __ddiv_rn(__dsub_rn(sigma[i * d + j], s), L[j * kMaxD + j]);
+        const double l = lane < DMAX ? sL[lane][k] : 0.0;
+#pragma unroll
+        for (int j = 0; j < kJ; ++j)
+          if (j > 0 || w > o) acc[j] = __fma_rn(l, sL[base + kW * j + w][k], acc[j]);
       }
     }
-  }
-  // P = L^-1 (lower triangular), column by column
-  for (int c = 0; c < d; ++c) {
-    for (int r = 0; r < d; ++r) {
-      double acc = (r == c) ? 1.0 : 0.0;
-      for (int k = c; k < r; ++k) acc -= L[r * kMaxD + k] * tg->P[k * kMaxD + c];
-      tg->P[r * kMaxD + c] = (r < c) ? 0.0 : acc / L[r * kMaxD + r];
+#pragma unroll
+    for (int j = 0; j < kJ; ++j) {
+      acc[j] = acc[j + 1];
+      row[j] = row[j + 1];
     }
   }
-  for (int i = 0; i < kMaxD * kMaxD; ++i) tg->Pf[i] = float(tg->P[i]);
+  __syncthreads();
+  if (lane < DMAX)
+    for (int r = w; r < d; r += kW) tg->L[r * kMaxD + lane] = sL[r][lane];
+  // P, lane = column: rows from the top, each finished row subtracted from
+  // the ones below; acc[j] is row base + 4 j + w
+#pragma unroll
+  for (int j = 0; j <= kJ; ++j) acc[j] = kW * j + w == lane ? 1.0 : 0.0;
+#pragma unroll 1
+  for (int base = 0; base < d; base += kW) {
+#pragma unroll
+    for (int o = 0; o < kW; ++o) {
+      const int k = base + o;
+      if (k < d) {
+        if (w == o) {
+          const double pk = (k < lane || lane >= d) ? 0.0 : __ddiv_rn(acc[0], sL[k][k]);
+          sp[lane] = pk;
+          if (lane < d) {
+            tg->P[k * kMaxD + lane] = pk;
+            tg->Pf[k * kMaxD + lane] = float(pk);
+          }
+        }
+        __syncthreads();
+        const double pk = sp[lane];
+#pragma unroll
+        for (int j = 0; j < kJ; ++j)
+          if (j > 0 || w > o) acc[j] = __fma_rn(-sL[base + kW * j + w][k], pk, acc[j]);
+        __syncthreads();  // (sp is read before the next row's)
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kJ; ++j) acc[j] = acc[j + 1];
+  }
 }
 
 // Logistic data: FP32 copies, BF16 hi / lo images of X log2(e) (the tensor-core
@@ -912,7 +978,14 @@ cudaError_t launch_particles(int op, const ParticleArgs& a, int grid, int thread
 
 cudaError_t launch_target_setup(TargetDev* tg, int kind, double nu, const double* mu, const double* sigma, int d,
                                 DevState* st, cudaStream_t s) {
-  k_target_setup<<<1, 32, 0, s>>>(tg, kind, nu, mu, sigma, d, st);
+  if (d <= 4)
+    k_target_setup<4><<<1, 32 * kSetupWarps, 0, s>>>(tg, kind, nu, mu, sigma, d, st);
+  else if (d <= 8)
+    k_target_setup<8><<<1, 32 * kSetupWarps, 0, s>>>(tg, kind, nu, mu, sigma, d, st);
+  else if (d <= 16)
+    k_target_setup<16><<<1, 32 * kSetupWarps, 0, s>>>(tg, kind, nu, mu, sigma, d, st);
+  else
+    k_target_setup<32><<<1, 32 * kSetupWarps, 0, s>>>(tg, kind, nu, mu, sigma, d, st);
   return cudaGetLastError();
 }
 
