@@ -1364,6 +1364,18 @@ __device__ __forceinline__ void load_counts(const int32_t* __restrict__ nc, int6
   }
 }
 
+// A block's sum of copy counts carries this bit when a count was negative.
+constexpr uint64_t kNcBad = 1ull << 63;
+
+// The outcome of the checks: SMC_EINVAL recorded, or (stateless calls, whose
+// error word starts with the call) set to what was found.
+__device__ __forceinline__ void nc_verdict(const NcScanArgs& a, bool bad) {
+  if (a.reset_err)
+    a.st->err = bad ? SMC_EINVAL : SMC_OK;
+  else if (bad)
+    record_error(a.st, SMC_EINVAL);
+}
+
 // Exclusive prefix of the block sums (cbase) and the check sum == n.
 __device__ __forceinline__ void nc_finalize_body(const NcScanArgs& a) {
   __shared__ uint64_t scratch[33];
@@ -1371,14 +1383,20 @@ __device__ __forceinline__ void nc_finalize_body(const NcScanArgs& a) {
   const int chunk = (nb + blockDim.x - 1) / blockDim.x;
   const int b0 = threadIdx.x * chunk, b1 = min(nb, b0 + chunk);
   uint64_t local = 0;
-  for (int b = b0; b < b1; ++b) local += a.part[b];
+  bool bad = false;
+  for (int b = b0; b < b1; ++b) {
+    const uint64_t v = a.part[b];
+    local += v & ~kNcBad;
+    bad |= (v & kNcBad) != 0;
+  }
   uint64_t total;
   uint64_t pre = block_excl_scan_u64(local, scratch, &total);
   for (int b = b0; b < b1; ++b) {
     a.cbase[b] = pre;
-    pre += a.part[b];
+    pre += a.part[b] & ~kNcBad;
   }
-  if (threadIdx.x == 0 && total != uint64_t(a.n)) record_error(a.st, SMC_EINVAL);
+  bad = __syncthreads_or(bad) || total != uint64_t(a.n);
+  if (threadIdx.x == 0) nc_verdict(a, bad);
 }
 
 __global__ void __launch_bounds__(kQThreads) k_nc_reduce(NcScanArgs a) {
@@ -1418,9 +1436,12 @@ __global__ void __launch_bounds__(kQThreads) k_nc_reduce(NcScanArgs a) {
   if (threadIdx.x == 0) {
     uint64_t t = 0;
     for (int w = 0; w < kQThreads / 32; ++w) t += sh[w];
-    a.part[blockIdx.x] = t;
-    if (bad) record_error(a.st, SMC_EINVAL);
+    a.part[blockIdx.x] = t | (bad ? kNcBad : 0);
   }
+  // (stamped calls: this block's share of the stamps, zero until the scan)
+  constexpr int kStamps = kQTile / kRTile;
+  if (a.stamps && threadIdx.x < kStamps && blockIdx.x * kStamps + threadIdx.x < a.ntiles)
+    a.stamps[blockIdx.x * kStamps + threadIdx.x] = 0;
 }
 
 __global__ void __launch_bounds__(kFinThreads) k_nc_finalize(NcScanArgs a) { nc_finalize_body(a); }
@@ -1533,6 +1554,105 @@ __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
     for (int k = threadIdx.x; w0 + uint64_t(k) < wend; k += blockDim.x) rs[k] = win[k];
     if (stamped && threadIdx.x < kNcWin / kRTile + 2 && s_has[threadIdx.x]) a.stamps[tfirst + threadIdx.x] = 1;
   }
+}
+
+// Up to kNcSmall blocks of counts: the three passes as one.  Every block reads
+// all counts (at most 512 KB from L2), so it knows its own prefix and the
+// total without a launch before it, and writes its whole output window, so
+// that no run start of an earlier call is left and no stamps are needed.
+// (n = 65537: 17 blocks, @@ us instead of 16 and two launches and two memsets more.)
+constexpr int kNcSmall = 32;
+
+__global__ void __launch_bounds__(kQThreads) k_nc_small(NcScanArgs a) {
+  __shared__ int32_t win[kNcWin];
+  __shared__ uint64_t scratch[33];
+  __shared__ uint64_t sh[kQThreads / 32][2];
+  __shared__ BigRuns big;
+  const int64_t n = a.n;
+  const uint64_t un = uint64_t(n);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (threadIdx.x == 0) big.count = 0;
+  int32_t c[kQItems];
+  uint64_t before = 0, total = 0, tsum = 0;
+  bool neg = false;
+  // (the sums only need every count once: coalesced 16-byte loads, eight in
+  // flight per thread; the block's own counts again, 16 per thread in order)
+  load_counts(a.ncopies, n, int64_t(blockIdx.x) * kQTile + int64_t(threadIdx.x) * kQItems, c);
+  const int64_t own = int64_t(blockIdx.x) * kQTile;
+  auto add = [&](int32_t v, int64_t i) {
+    neg |= v < 0;
+    const uint32_t u = uint32_t(max(v, 0));
+    total += u;
+    if (i < own) before += u;
+  };
+  int64_t done = 0;
+  if ((reinterpret_cast<uintptr_t>(a.ncopies) & 15) == 0) {
+    const int4* p = reinterpret_cast<const int4*>(a.ncopies);
+    const int n4 = int(n / 4);
+    for (int e = threadIdx.x; e < n4; e += 8 * kQThreads) {
+      int4 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = e + u * kQThreads;
+        v[u] = k < n4 ? __ldg(p + k) : make_int4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int64_t i = 4 * int64_t(e + u * kQThreads);  // (a tile starts at a multiple of 4)
+        neg |= (v[u].x | v[u].y | v[u].z | v[u].w) < 0;
+        const uint64_t t = uint64_t(uint32_t(max(v[u].x, 0))) + uint32_t(max(v[u].y, 0)) + uint32_t(max(v[u].z, 0)) +
+                           uint32_t(max(v[u].w, 0));
+        total += t;
+        if (i < own) before += t;
+      }
+    }
+    done = 4 * int64_t(n4);
+  }
+  for (int64_t i = done + threadIdx.x; i < n; i += kQThreads) add(a.ncopies[i], i);
+#pragma unroll
+  for (int q = 0; q < kQItems; ++q) tsum += uint32_t(max(c[q], 0));
+  before = warp_sum(before);
+  total = warp_sum(total);
+  if (lane == 0) {
+    sh[wid][0] = before;
+    sh[wid][1] = total;
+  }
+  neg = __syncthreads_or(neg);
+  uint64_t w0 = 0;
+  total = 0;
+  for (int w = 0; w < kQThreads / 32; ++w) {
+    w0 += sh[w][0];
+    total += sh[w][1];
+  }
+  const bool bad = neg || total != un;
+  if (blockIdx.x == 0 && threadIdx.x == 0) nc_verdict(a, bad);
+  if (bad || (!a.reset_err && a.st->err)) return;
+  uint64_t btot;
+  const uint64_t excl = block_excl_scan_u64(tsum, scratch, &btot);
+  const bool staged = btot <= uint64_t(kNcWin);
+  int32_t* __restrict__ rs = rs_now(a.runstart, a.runstart_alt, a.st) + w0;
+  if (staged) {
+    for (int k = threadIdx.x; k < int(btot); k += blockDim.x) win[k] = -1;
+  } else {
+    for (uint64_t k = threadIdx.x; k < btot; k += blockDim.x) rs[k] = -1;
+  }
+  __syncthreads();  // every -1 before any run start
+  uint64_t o = excl;
+  const int64_t i0 = int64_t(blockIdx.x) * kQTile + int64_t(threadIdx.x) * kQItems;
+#pragma unroll
+  for (int q = 0; q < kQItems; ++q) {
+    if (c[q] > 0) {
+      if (staged)
+        win[o] = int32_t(i0 + q);
+      else
+        rs[o] = int32_t(i0 + q);
+      tile_starts_of_run(a.tile_src, w0 + o, w0 + o + uint32_t(c[q]), un, int32_t(i0 + q), big);
+      o += uint32_t(c[q]);
+    }
+  }
+  tile_starts_flush(a.tile_src, big);  // (block barrier inside)
+  if (staged)
+    for (int k = threadIdx.x; k < int(btot); k += blockDim.x) rs[k] = win[k];
 }
 
 // ---------------------------------------------------------------- redistribute
@@ -2001,17 +2121,15 @@ cudaError_t launch_iter_scan(const QuantArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_nc_reduce(const NcScanArgs& a, cudaStream_t s) {
+bool nc_small(int64_t n) { return qblocks(n) <= kNcSmall; }
+
+cudaError_t launch_nc(const NcScanArgs& a, cudaStream_t s) {
+  if (nc_small(a.n)) {
+    k_nc_small<<<qblocks(a.n), kQThreads, 0, s>>>(a);
+    return cudaGetLastError();
+  }
   k_nc_reduce<<<qblocks(a.n), kQThreads, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_nc_finalize(const NcScanArgs& a, cudaStream_t s) {
   k_nc_finalize<<<1, kFinThreads, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_nc_scan(const NcScanArgs& a, cudaStream_t s) {
   k_nc_scan<<<qblocks(a.n), kQThreads, 0, s>>>(a);
   return cudaGetLastError();
 }

@@ -558,9 +558,7 @@ int smc_redistribute(smc_sampler* h, const int32_t* ncopies_dev) {
   s.nblocks = h->L.qblocks;
   s.ntiles = h->L.ntiles;
   s.st = h->st;
-  SMC_TRY(h, launch_nc_reduce(s, h->stream));
-  SMC_TRY(h, launch_nc_finalize(s, h->stream));
-  SMC_TRY(h, launch_nc_scan(s, h->stream));
+  SMC_TRY(h, launch_nc(s, h->stream));
   SMC_TRY(h, launch_redistribute(redist_args(h, 1), h->stream));
   SMC_TRY(h, launch_commit(h->st, h->d, 1, 0, h->stream));
   return SMC_OK;
@@ -770,7 +768,8 @@ int redistribute_raw_impl(int64_t n, int32_t row_bytes, const int32_t* ncopies_d
   a.st = st;
   // stamped: the run-start array is not cleared; the copy reads the slices
   // of the stamped tiles only, which the scan writes whole
-  a.stamps = reinterpret_cast<int32_t*>(ws + L.stamps);
+  a.stamps = nc_small(n) ? nullptr : reinterpret_cast<int32_t*>(ws + L.stamps);
+  a.reset_err = 1;
   RedistArgs r{};
   r.n = n;
   r.row_bytes = row_bytes;
@@ -786,11 +785,7 @@ int redistribute_raw_impl(int64_t n, int32_t row_bytes, const int32_t* ncopies_d
   r.stateful = 0;
   r.stamps = a.stamps;
   cudaError_t e = rec(0);
-  if (e == cudaSuccess) e = cudaMemsetAsync(&st->err, 0, sizeof(int32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(a.stamps, 0, size_t(L.ntiles) * sizeof(int32_t), s);
-  if (e == cudaSuccess) e = launch_nc_reduce(a, s);
-  if (e == cudaSuccess) e = launch_nc_finalize(a, s);
-  if (e == cudaSuccess) e = launch_nc_scan(a, s);
+  if (e == cudaSuccess) e = launch_nc(a, s);
   if (e == cudaSuccess) e = rec(1);
   if (e == cudaSuccess) e = launch_redistribute(r, s);
   if (e == cudaSuccess) e = rec(2);

@@ -181,11 +181,11 @@ struct NcScanArgs {
   int32_t ntiles;
   DevState* st;
   int32_t clear_rs;     // the reduce pass sets runstart[0, n) to -1 first (runstart_alt NULL)
-  int32_t pad;
-  // stamped calls (the stateless entry points; zeroed by the caller before
-  // each call): per copy tile, set when a run start lands in it -- runstart
+  int32_t reset_err;    // 1: the error word is this call's (set to its outcome); 0: an error is added to it
+  // stamped calls (the stateless entry points above nc_small; zeroed by the
+  // reduce pass): per kRTile output rows, set when a run start lands in them -- runstart
   // then need not be clean on entry (k_nc_scan writes every slice the copy
-  // reads); NULL: runstart must hold -1 everywhere on entry
+  // reads); NULL: runstart must hold -1 everywhere on entry (above nc_small)
   int32_t* stamps;
 };
 
@@ -255,9 +255,8 @@ cudaError_t launch_quant_scan(const QuantArgs& a, cudaStream_t s);
 // scan with the iteration's statistics in one more block
 cudaError_t launch_iter_finalize(const QuantArgs& a, cudaStream_t s);
 cudaError_t launch_iter_scan(const QuantArgs& a, cudaStream_t s);
-cudaError_t launch_nc_reduce(const NcScanArgs& a, cudaStream_t s);
-cudaError_t launch_nc_finalize(const NcScanArgs& a, cudaStream_t s);
-cudaError_t launch_nc_scan(const NcScanArgs& a, cudaStream_t s);
+bool nc_small(int64_t n);  // the scan writes every run start itself: no stamps at this size
+cudaError_t launch_nc(const NcScanArgs& a, cudaStream_t s);  // exclusive scan of ncopies: run starts, tile sources
 cudaError_t launch_redistribute(const RedistArgs& a, cudaStream_t s);
 // fused small samplers (N <= kSmallTile): redistribute + commit as one launch
 cudaError_t launch_redistribute_commit(const RedistArgs& a, int d, int force_flip, int recycle, cudaStream_t s);

@@ -109,6 +109,7 @@ extern "C" int smc_redistribute_raw_noalloc(int64_t n, int32_t row_bytes, const 
   a.nblocks = int32_t((n + kQTile - 1) / kQTile);
   a.ntiles = int32_t((n + kRTile - 1) / kRTile);
   a.st = st;
+  a.reset_err = 1;
   RedistArgs r{};
   r.n = n;
   r.row_bytes = row_bytes;
@@ -122,10 +123,7 @@ extern "C" int smc_redistribute_raw_noalloc(int64_t n, int32_t row_bytes, const 
   r.logw = nullptr;
   r.st = st;
   r.stateful = 0;
-  e = cudaMemsetAsync(&st->err, 0, sizeof(int32_t), s);
-  if (e == cudaSuccess) e = launch_nc_reduce(a, s);
-  if (e == cudaSuccess) e = launch_nc_finalize(a, s);
-  if (e == cudaSuccess) e = launch_nc_scan(a, s);
+  e = launch_nc(a, s);
   if (e == cudaSuccess) e = launch_redistribute(r, s);
   if (e == cudaSuccess && status_dev)
     e = cudaMemcpyAsync(status_dev, &st->err, sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
