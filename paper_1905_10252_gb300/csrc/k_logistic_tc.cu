@@ -215,6 +215,7 @@ __device__ __forceinline__ void add_exact(float v, float& hi, float& lo) {
 }
 
 __global__ void __launch_bounds__(kTcThreads, 1) k_logistic_tc(ParticleArgs a) {
+  chain_begin();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* xs = sm;                                   // kTcStages x (hi | lo) half tiles
@@ -613,7 +614,7 @@ cudaError_t launch_logistic_tc(const ParticleArgs& a, int grid, cudaStream_t s) 
     if (e != cudaSuccess) return e;
     configured[dev].store(true);
   }
-  k_logistic_tc<<<grid, kTcThreads, kTcSmem, s>>>(a);
+  chain_launch(k_logistic_tc, grid, kTcThreads, kTcSmem, s, a);
   return cudaGetLastError();
 }
 

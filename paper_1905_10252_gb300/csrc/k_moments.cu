@@ -110,6 +110,7 @@ template <typename T>
 __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const double* cov,
                                                       double* __restrict__ covpart,
                                                       const uint64_t* __restrict__ exp_table) {
+  chain_begin();
   using S = CovShape<T>;
   constexpr bool kF32 = sizeof(T) == 4;
   if (!cov) cov = a.st->cov_out;
@@ -327,6 +328,7 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
 // addition after another: 42 us.)
 __global__ void __launch_bounds__(128) k_cov_finalize(const DevState* st, double* cov,
                                                      const double* __restrict__ covpart, int nblocks, int d) {
+  chain_begin();
   if (!cov) cov = st->cov_out;
   if (!cov || st->err) return;
   const int npairs = d * (d + 1) / 2;
@@ -354,13 +356,13 @@ cudaError_t launch_cov(const ParticleArgs& a, double* cov, double* covpart, int 
   cudaError_t e = expfx_table(&table);
   if (e != cudaSuccess) return e;
   if (a.dtype == SMC_F64)
-    k_cov<double><<<grid, kCovThreads, 0, s>>>(a, cov, covpart, table);
+    chain_launch(k_cov<double>, grid, kCovThreads, 0, s, a, cov, covpart, table);
   else
-    k_cov<float><<<grid, kCovThreads, 0, s>>>(a, cov, covpart, table);
+    chain_launch(k_cov<float>, grid, kCovThreads, 0, s, a, cov, covpart, table);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int npairs = a.d * (a.d + 1) / 2;
-  k_cov_finalize<<<(npairs + 3) / 4, 128, 0, s>>>(a.st, cov, covpart, grid, a.d);
+  chain_launch(k_cov_finalize, (npairs + 3) / 4, 128, 0, s, a.st, cov, covpart, grid, a.d);
   return cudaGetLastError();
 }
 

@@ -262,6 +262,7 @@ __global__ void __launch_bounds__(kPThreads) k_init(ParticleArgs a) {
 // FP32 targets): move_reweight_generic_body over the whole launch.
 template <typename T, int DMAX, bool MOVE, bool REWEIGHT>
 __global__ void __launch_bounds__(kPThreads) k_move_reweight(ParticleArgs a) {
+  chain_begin();
   __shared__ TargetSmem<T> ts;
   move_reweight_generic_body<T, DMAX, MOVE, REWEIGHT>(a, ts, blockIdx.x, gridDim.x, blockDim.x,
                                                       (a.flags & PA_FUSED_ITER) ? 1 : 0);
@@ -786,6 +787,7 @@ __device__ __forceinline__ void move_reweight_body(const ParticleArgs& a, const 
 // the FMAs straight from the constant bank.
 template <int DPL, bool MOVE, bool REWEIGHT, bool EST = false, bool GATHER = false, bool FULL = false>
 __global__ void __launch_bounds__(kPThreads, 2) k_move_reweight_lanes(ParticleArgs a, const GaussParamsF32 gp) {
+  chain_begin();
   move_reweight_body<DPL, MOVE, REWEIGHT, FactorParam, EST, GATHER, FULL>(a, FactorParam{gp}, blockIdx.x, gridDim.x);
 }
 
@@ -906,9 +908,9 @@ template <typename T, int DMAX>
 static cudaError_t launch_particles_t(int op, const ParticleArgs& a, int grid, int threads, cudaStream_t s) {
   switch (op) {
     case OP_INIT: k_init<T, DMAX><<<grid, threads, 0, s>>>(a); break;
-    case OP_MOVE: k_move_reweight<T, DMAX, true, false><<<grid, threads, 0, s>>>(a); break;
-    case OP_REWEIGHT: k_move_reweight<T, DMAX, false, true><<<grid, threads, 0, s>>>(a); break;
-    case OP_MOVE_REWEIGHT: k_move_reweight<T, DMAX, true, true><<<grid, threads, 0, s>>>(a); break;
+    case OP_MOVE: chain_launch(k_move_reweight<T, DMAX, true, false>, grid, threads, 0, s, a); break;
+    case OP_REWEIGHT: chain_launch(k_move_reweight<T, DMAX, false, true>, grid, threads, 0, s, a); break;
+    case OP_MOVE_REWEIGHT: chain_launch(k_move_reweight<T, DMAX, true, true>, grid, threads, 0, s, a); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -931,20 +933,20 @@ static cudaError_t launch_lanes(int op, const ParticleArgs& a, int grid, int thr
                                 const GaussParamsF32& gp) {
   const bool full = a.d == DPL;
   switch (op) {
-    case OP_MOVE: k_move_reweight_lanes<DPL, true, false><<<grid, threads, 0, s>>>(a, gp); break;
-    case OP_REWEIGHT: k_move_reweight_lanes<DPL, false, true><<<grid, threads, 0, s>>>(a, gp); break;
+    case OP_MOVE: chain_launch(k_move_reweight_lanes<DPL, true, false>, grid, threads, 0, s, a, gp); break;
+    case OP_REWEIGHT: chain_launch(k_move_reweight_lanes<DPL, false, true>, grid, threads, 0, s, a, gp); break;
     case OP_MOVE_REWEIGHT:
       if (full)
-        k_move_reweight_lanes<DPL, true, true, false, false, true><<<grid, threads, 0, s>>>(a, gp);
+        chain_launch(k_move_reweight_lanes<DPL, true, true, false, false, true>, grid, threads, 0, s, a, gp);
       else
-        k_move_reweight_lanes<DPL, true, true><<<grid, threads, 0, s>>>(a, gp);
+        chain_launch(k_move_reweight_lanes<DPL, true, true>, grid, threads, 0, s, a, gp);
       break;
     case OP_MOVE_REWEIGHT_EST:  // D <= 16 only (register room)
       if constexpr (DPL <= 16) {
         if (full)
-          k_move_reweight_lanes<DPL, true, true, true, false, true><<<grid, threads, 0, s>>>(a, gp);
+          chain_launch(k_move_reweight_lanes<DPL, true, true, true, false, true>, grid, threads, 0, s, a, gp);
         else
-          k_move_reweight_lanes<DPL, true, true, true><<<grid, threads, 0, s>>>(a, gp);
+          chain_launch(k_move_reweight_lanes<DPL, true, true, true>, grid, threads, 0, s, a, gp);
         break;
       } else {
         return cudaErrorInvalidValue;
@@ -952,9 +954,9 @@ static cudaError_t launch_lanes(int op, const ParticleArgs& a, int grid, int thr
     case OP_MOVE_REWEIGHT_GATHER:  // (the same, and gathers a pending resampling's rows)
       if constexpr (DPL <= 16) {
         if (full)
-          k_move_reweight_lanes<DPL, true, true, true, true, true><<<grid, threads, 0, s>>>(a, gp);
+          chain_launch(k_move_reweight_lanes<DPL, true, true, true, true, true>, grid, threads, 0, s, a, gp);
         else
-          k_move_reweight_lanes<DPL, true, true, true, true><<<grid, threads, 0, s>>>(a, gp);
+          chain_launch(k_move_reweight_lanes<DPL, true, true, true, true>, grid, threads, 0, s, a, gp);
         break;
       } else {
         return cudaErrorInvalidValue;

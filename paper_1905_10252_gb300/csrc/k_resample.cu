@@ -103,6 +103,7 @@ __device__ __forceinline__ void load_table(uint64_t* T) {
 // reset value of Algorithm 4 line 3, -log N, from the exact log so that both
 // implementations agree bit for bit
 __global__ void k_state_init(DevState* st, int64_t n, int64_t t, int F) {
+  chain_begin();
   if (threadIdx.x != 0) return;
   const double reset_logw = -det_log(double(n));
   st->t = t;
@@ -143,6 +144,7 @@ __global__ void k_state_init(DevState* st, int64_t n, int64_t t, int F) {
 // thread in flight: FP64 comparisons and a count (two lanes per SM and clock
 // each) took 155 us at N = 2^24, 27 now.
 __global__ void __launch_bounds__(kQThreads) k_max_logw(const double* __restrict__ logw, int64_t n, DevState* st) {
+  chain_begin();
   __shared__ long long shm[kQThreads / 32];
   MaxTracker mt;
   mt.init();
@@ -489,6 +491,7 @@ __device__ __forceinline__ void quant_reduce_body(const QuantArgs& a, const int 
 
 template <typename ST, int DMAX, bool EST>
 __global__ void __launch_bounds__(kQThreads) k_quant_reduce(QuantArgs a) {
+  chain_begin();
   __shared__ QuantReduceSmem sm;
   quant_reduce_body<ST, DMAX, EST>(a, blockIdx.x, sm);
 }
@@ -564,6 +567,7 @@ __device__ __forceinline__ void load_cols(const double* __restrict__ row, int c,
 
 template <typename ST, int CW, bool EST>
 __global__ void __launch_bounds__(kQThreads, 2) __cluster_dims__(kQSplit, 1, 1) k_quant_reduce_cluster(QuantArgs a) {
+  chain_begin();
   __shared__ QuantClusterSmem sm;
   const int s = int(cluster_rank());
   const int64_t tile = blockIdx.x / kQSplit;
@@ -928,6 +932,7 @@ __global__ void __launch_bounds__(kFinThreads) k_quant_finalize(QuantArgs a, int
 // kernels, with the logarithm and divisions of the statistics in the chain,
 // these steps took 22 us of an iteration whatever N.
 __global__ void __launch_bounds__(kFinThreads) k_iter_finalize(QuantArgs a) {
+  chain_begin();
   __shared__ uint64_t s_w[33], s_2l[32], s_2h[32], s_el[32], s_eh[32];
   DevState* st = a.st;
   const int nb = a.nblocks, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
@@ -1324,6 +1329,7 @@ __global__ void __launch_bounds__(kQThreads, 4) k_quant_scan_sub(QuantArgs a) {
 // it: as the last block they ended a scan of 4096 blocks 10 us later).
 template <bool SUB>
 __global__ void __launch_bounds__(kQThreads, 4) k_iter_scan(QuantArgs a) {
+  chain_begin();
   __shared__ union {
     ScanSmem scan;
     IterStatsSmem stats;
@@ -1400,6 +1406,7 @@ __device__ __forceinline__ void nc_finalize_body(const NcScanArgs& a) {
 }
 
 __global__ void __launch_bounds__(kQThreads) k_nc_reduce(NcScanArgs a) {
+  chain_begin();
   __shared__ uint64_t sh[kQThreads / 32];
   __shared__ int bad;
   if (threadIdx.x == 0) bad = 0;
@@ -1444,7 +1451,7 @@ __global__ void __launch_bounds__(kQThreads) k_nc_reduce(NcScanArgs a) {
     a.stamps[blockIdx.x * kStamps + threadIdx.x] = 0;
 }
 
-__global__ void __launch_bounds__(kFinThreads) k_nc_finalize(NcScanArgs a) { nc_finalize_body(a); }
+__global__ void __launch_bounds__(kFinThreads) k_nc_finalize(NcScanArgs a) { chain_begin(); nc_finalize_body(a); }
 
 // Run starts of the block's items.  The block's outputs form the window
 // [cbase, cbase + total); the windows of the blocks are disjoint and tile
@@ -1464,6 +1471,7 @@ constexpr int kFillTiles = 1024;
 constexpr uint64_t kFillAll = 1u << 17;
 
 __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
+  chain_begin();
   if (a.st->err) return;
   __shared__ int32_t win[kNcWin];
   __shared__ uint64_t scratch[33];
@@ -1564,6 +1572,7 @@ __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
 constexpr int kNcSmall = 32;
 
 __global__ void __launch_bounds__(kQThreads) k_nc_small(NcScanArgs a) {
+  chain_begin();
   __shared__ int32_t win[kNcWin];
   __shared__ uint64_t scratch[33];
   __shared__ uint64_t sh[kQThreads / 32][2];
@@ -1780,6 +1789,7 @@ __device__ __forceinline__ void redistribute_body(const RedistArgs& a, const int
 
 template <typename V, int CPR, int TILE>
 __global__ void __launch_bounds__(kRThreads) k_redistribute(RedistArgs a) {
+  chain_begin();
   __shared__ RedistSmemT<TILE> sm;
   redistribute_body<V, CPR, 8, false, TILE>(a, blockIdx.x, sm);
   if (a.end_iter) end_iteration(a.st, gridDim.x, 0);
@@ -2045,12 +2055,12 @@ cudaError_t launch_identity_runs_batch(const RedistArgs* ra, const int4* map, in
 static int qblocks(int64_t n) { return int((n + kQTile - 1) / kQTile); }
 
 cudaError_t launch_state_init(DevState* st, int64_t n, int64_t t, int F, cudaStream_t s) {
-  k_state_init<<<1, 32, 0, s>>>(st, n, t, F);
+  chain_launch(k_state_init, 1, 32, 0, s, st, n, t, F);
   return cudaGetLastError();
 }
 
 cudaError_t launch_max_logw(const double* logw, int64_t n, DevState* st, cudaStream_t s) {
-  k_max_logw<<<qblocks(n), kQThreads, 0, s>>>(logw, n, st);
+  chain_launch(k_max_logw, qblocks(n), kQThreads, 0, s, logw, n, st);
   return cudaGetLastError();
 }
 
@@ -2070,23 +2080,23 @@ static cudaError_t quant_reduce_t(const QuantArgs& a, cudaStream_t s) {
   const bool est = a.x[0] && a.d >= 1;
   if (quant_split(a.n)) {
     if (!est)
-      k_quant_reduce_cluster<ST, 1, false><<<g * kQSplit, kQThreads, 0, s>>>(a);
+      chain_launch(k_quant_reduce_cluster<ST, 1, false>, g * kQSplit, kQThreads, 0, s, a);
     else if (a.d <= 8)
-      k_quant_reduce_cluster<ST, 1, true><<<g * kQSplit, kQThreads, 0, s>>>(a);
+      chain_launch(k_quant_reduce_cluster<ST, 1, true>, g * kQSplit, kQThreads, 0, s, a);
     else if (a.d <= 16)
-      k_quant_reduce_cluster<ST, 2, true><<<g * kQSplit, kQThreads, 0, s>>>(a);
+      chain_launch(k_quant_reduce_cluster<ST, 2, true>, g * kQSplit, kQThreads, 0, s, a);
     else
-      k_quant_reduce_cluster<ST, 4, true><<<g * kQSplit, kQThreads, 0, s>>>(a);
+      chain_launch(k_quant_reduce_cluster<ST, 4, true>, g * kQSplit, kQThreads, 0, s, a);
   } else if (!est) {
-    k_quant_reduce<ST, 1, false><<<g, kQThreads, 0, s>>>(a);
+    chain_launch(k_quant_reduce<ST, 1, false>, g, kQThreads, 0, s, a);
   } else if (a.d <= 4) {
-    k_quant_reduce<ST, 4, true><<<g, kQThreads, 0, s>>>(a);
+    chain_launch(k_quant_reduce<ST, 4, true>, g, kQThreads, 0, s, a);
   } else if (a.d <= 8) {
-    k_quant_reduce<ST, 8, true><<<g, kQThreads, 0, s>>>(a);
+    chain_launch(k_quant_reduce<ST, 8, true>, g, kQThreads, 0, s, a);
   } else if (a.d <= 16) {
-    k_quant_reduce<ST, 16, true><<<g, kQThreads, 0, s>>>(a);
+    chain_launch(k_quant_reduce<ST, 16, true>, g, kQThreads, 0, s, a);
   } else {
-    k_quant_reduce<ST, 32, true><<<g, kQThreads, 0, s>>>(a);
+    chain_launch(k_quant_reduce<ST, 32, true>, g, kQThreads, 0, s, a);
   }
   return cudaGetLastError();
 }
@@ -2109,15 +2119,15 @@ cudaError_t launch_quant_scan(const QuantArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_iter_finalize(const QuantArgs& a, cudaStream_t s) {
-  k_iter_finalize<<<1, a.nblocks > 256 ? kFinThreads : 256, 0, s>>>(a);
+  chain_launch(k_iter_finalize, 1, a.nblocks > 256 ? kFinThreads : 256, 0, s, a);
   return cudaGetLastError();
 }
 
 cudaError_t launch_iter_scan(const QuantArgs& a, cudaStream_t s) {
   if (quant_split(a.n))
-    k_iter_scan<true><<<qblocks(a.n) * kQSplit + 1, kQThreads, 0, s>>>(a);
+    chain_launch(k_iter_scan<true>, qblocks(a.n) * kQSplit + 1, kQThreads, 0, s, a);
   else
-    k_iter_scan<false><<<qblocks(a.n) + 1, kQThreads, 0, s>>>(a);
+    chain_launch(k_iter_scan<false>, qblocks(a.n) + 1, kQThreads, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -2125,12 +2135,12 @@ bool nc_small(int64_t n) { return qblocks(n) <= kNcSmall; }
 
 cudaError_t launch_nc(const NcScanArgs& a, cudaStream_t s) {
   if (nc_small(a.n)) {
-    k_nc_small<<<qblocks(a.n), kQThreads, 0, s>>>(a);
+    chain_launch(k_nc_small, qblocks(a.n), kQThreads, 0, s, a);
     return cudaGetLastError();
   }
-  k_nc_reduce<<<qblocks(a.n), kQThreads, 0, s>>>(a);
-  k_nc_finalize<<<1, kFinThreads, 0, s>>>(a);
-  k_nc_scan<<<qblocks(a.n), kQThreads, 0, s>>>(a);
+  chain_launch(k_nc_reduce, qblocks(a.n), kQThreads, 0, s, a);
+  chain_launch(k_nc_finalize, 1, kFinThreads, 0, s, a);
+  chain_launch(k_nc_scan, qblocks(a.n), kQThreads, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -2142,22 +2152,22 @@ static void redistribute_t(const RedistArgs& a, cudaStream_t s) {
   const int rb = a.row_bytes;
   if (rb % 16 == 0) {
     switch (rb / 16) {
-      case 1: k_redistribute<uint4, 1, TILE><<<grid, kRThreads, 0, s>>>(a); break;
-      case 2: k_redistribute<uint4, 2, TILE><<<grid, kRThreads, 0, s>>>(a); break;
-      case 4: k_redistribute<uint4, 4, TILE><<<grid, kRThreads, 0, s>>>(a); break;
-      case 8: k_redistribute<uint4, 8, TILE><<<grid, kRThreads, 0, s>>>(a); break;
-      default: k_redistribute<uint4, 0, TILE><<<grid, kRThreads, 0, s>>>(a); break;
+      case 1: chain_launch(k_redistribute<uint4, 1, TILE>, grid, kRThreads, 0, s, a); break;
+      case 2: chain_launch(k_redistribute<uint4, 2, TILE>, grid, kRThreads, 0, s, a); break;
+      case 4: chain_launch(k_redistribute<uint4, 4, TILE>, grid, kRThreads, 0, s, a); break;
+      case 8: chain_launch(k_redistribute<uint4, 8, TILE>, grid, kRThreads, 0, s, a); break;
+      default: chain_launch(k_redistribute<uint4, 0, TILE>, grid, kRThreads, 0, s, a); break;
     }
   } else if (rb % 8 == 0) {
     if (rb == 8)
-      k_redistribute<uint2, 1, TILE><<<grid, kRThreads, 0, s>>>(a);
+      chain_launch(k_redistribute<uint2, 1, TILE>, grid, kRThreads, 0, s, a);
     else
-      k_redistribute<uint2, 0, TILE><<<grid, kRThreads, 0, s>>>(a);
+      chain_launch(k_redistribute<uint2, 0, TILE>, grid, kRThreads, 0, s, a);
   } else {
     if (rb == 4)
-      k_redistribute<uint32_t, 1, TILE><<<grid, kRThreads, 0, s>>>(a);
+      chain_launch(k_redistribute<uint32_t, 1, TILE>, grid, kRThreads, 0, s, a);
     else
-      k_redistribute<uint32_t, 0, TILE><<<grid, kRThreads, 0, s>>>(a);
+      chain_launch(k_redistribute<uint32_t, 0, TILE>, grid, kRThreads, 0, s, a);
   }
 }
 

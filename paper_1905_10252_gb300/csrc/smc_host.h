@@ -57,8 +57,10 @@ struct smc_sampler {
   // FP64 sampler of one quantise block and one copy tile: smc_step runs its
   // iterations in one cooperative launch (k_iterate_small)
   bool small_iter;
-  // CUDA graph of one iteration (with and without the covariance stage)
+  // CUDA graphs of one and of several iterations (without the covariance
+  // stage), and the iterations run by plain launches so far (smc_step)
   cudaGraphExec_t g_iter[2];
+  int plain_run;
   std::string err;
 };
 
