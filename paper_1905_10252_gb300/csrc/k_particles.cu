@@ -818,6 +818,29 @@ __global__ void __launch_bounds__(kPThreads, 2) k_move_reweight_batch(const Part
     move_reweight_body<32, true, true, FactorSmem, false>(a, fs, m.y, m.z);
 }
 
+// The same for a batch whose map is sorted by width class: one launch per
+// class (up to 8, 16, 32 coordinates, and exactly as many), each with its own
+// registers.  In one kernel for all classes the widest class's
+// registers left no room for the D-exact ones (they spilled).  The launches
+// after the first start while it runs (their inputs are complete when the
+// first starts) and end after it: their last act is to wait for the launch
+// before them, so that whatever follows the last follows all.
+template <int DPL, bool FULL>
+__global__ void __launch_bounds__(kPThreads, 2) k_move_reweight_class(const ParticleArgs* __restrict__ pa,
+                                                                     const GaussParamsF32* __restrict__ gps,
+                                                                     const int4* __restrict__ map) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int4 m = map[blockIdx.x];
+  const ParticleArgs a = pa[m.x];
+  __shared__ float4 sfac[kPairedFactor / 2];
+  __shared__ float smu[kTgtMaxD];
+  stage_pairs(gps[m.x].P2, gps[m.x].mu, a.d, reinterpret_cast<float2*>(sfac), smu);
+  __syncthreads();
+  const FactorSmem fs{sfac, smu};
+  move_reweight_body<DPL, true, true, FactorSmem, DPL <= 16, false, FULL>(a, fs, m.y, m.z);
+  if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- finalise the maximum
 // (max_finalize_body: particle_bodies.cuh)
 __global__ void __launch_bounds__(kFinThreads) k_max_finalize(const double* __restrict__ part, int nb,
@@ -1009,6 +1032,30 @@ cudaError_t launch_move_reweight_batch(const ParticleArgs* pa, const GaussParams
                                        cudaStream_t s, const int32_t* left) {
   k_move_reweight_batch<<<nblocks, kPThreads, 0, s>>>(pa, gps, map, left);
   return cudaGetLastError();
+}
+cudaError_t launch_move_reweight_classes(const ParticleArgs* pa, const GaussParamsF32* gps, const int4* map,
+                                         const int (&blocks)[kMoveClasses], cudaStream_t s) {
+  // (the first launch follows what is before it completely)
+  bool first = true;
+  cudaError_t e = cudaSuccess;
+  auto one = [&](auto kernel, int n) {
+    if (n == 0 || e != cudaSuccess) return;
+    if (first) {
+      kernel<<<n, kPThreads, 0, s>>>(pa, gps, map);
+      e = cudaGetLastError();
+    } else {
+      e = chain_launch(kernel, n, kPThreads, 0, s, pa, gps, map);
+    }
+    first = false;
+    map += n;
+  };
+  one(k_move_reweight_class<32, true>, blocks[0]);
+  one(k_move_reweight_class<32, false>, blocks[1]);
+  one(k_move_reweight_class<16, true>, blocks[2]);
+  one(k_move_reweight_class<16, false>, blocks[3]);
+  one(k_move_reweight_class<8, true>, blocks[4]);
+  one(k_move_reweight_class<8, false>, blocks[5]);
+  return e;
 }
 cudaError_t launch_max_finalize_batch(const ParticleArgs* pa, const int* nb, int count, cudaStream_t s,
                                       const int32_t* left) {

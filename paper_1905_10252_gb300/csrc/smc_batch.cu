@@ -34,7 +34,8 @@ struct Plan {
   int count = 0;
   std::vector<int4> qmap;                               // quantise / scan blocks
   std::vector<int4> rmap;                               // copy tiles
-  std::vector<int4> mmap[SMC_BATCH_MOVE_VARIANTS];      // move / reweight blocks
+  std::vector<int4> mmap[SMC_BATCH_MOVE_VARIANTS];      // move / reweight blocks, widest class first
+  int mblocks[SMC_BATCH_MOVE_VARIANTS][kMoveClasses] = {};  // of them per width class
   std::vector<int32_t> nb[SMC_BATCH_MOVE_VARIANTS];     // move blocks per member
 };
 
@@ -71,8 +72,12 @@ Plan make_plan(smc_sampler* const* m, int count, int sms) {
       if (kMoveBudget[v] > 0) b = int(std::llround(total * w[s] / wsum));
       p.nb[v][s] = std::max(1, std::min(b, full));
     }
-    for (int s : order)
-      for (int j = 0; j < p.nb[v][s]; ++j) p.mmap[v].push_back(make_int4(s, j, p.nb[v][s], 0));
+    for (int c = 0; c < kMoveClasses; ++c)
+      for (int s : order) {
+        if (move_class(m[s]->d) != c) continue;
+        for (int j = 0; j < p.nb[v][s]; ++j) p.mmap[v].push_back(make_int4(s, j, p.nb[v][s], 0));
+        p.mblocks[v][c] += p.nb[v][s];
+      }
   }
   return p;
 }
@@ -179,8 +184,8 @@ cudaError_t launch_batch_iteration(const smc_batch* b) {
   const int nq = int(b->plan.qmap.size());
   cudaError_t e = launch_begin_batch(pa, c, s);
   if (e == cudaSuccess)
-    e = launch_move_reweight_batch(pa, b->at<GaussParamsF32>(b->L.gp), b->at<int4>(b->L.mmap[mv]),
-                                   int(b->plan.mmap[mv].size()), s);
+    e = launch_move_reweight_classes(pa, b->at<GaussParamsF32>(b->L.gp), b->at<int4>(b->L.mmap[mv]),
+                                     b->plan.mblocks[mv], s);
   if (e == cudaSuccess) e = launch_max_finalize_batch(pa, b->at<int32_t>(b->L.nb) + size_t(mv) * c, c, s);
   if (e == cudaSuccess) e = launch_quant_reduce_batch(qa, qmap, nq, s);
   if (e == cudaSuccess) e = launch_quant_finalize_batch(qa, c, s);
@@ -384,8 +389,8 @@ int smc_batch_step_profile(smc_batch* b, void* const* events_host, int32_t n_eve
   BATCH_TRY(b, launch_step_setup_batch(pa, b->at<void*>(b->L.outs), c, s));
   BATCH_TRY(b, rec(0));
   BATCH_TRY(b, launch_begin_batch(pa, c, s));
-  BATCH_TRY(b, launch_move_reweight_batch(pa, b->at<GaussParamsF32>(b->L.gp), b->at<int4>(b->L.mmap[mv]),
-                                          int(b->plan.mmap[mv].size()), s));
+  BATCH_TRY(b, launch_move_reweight_classes(pa, b->at<GaussParamsF32>(b->L.gp), b->at<int4>(b->L.mmap[mv]),
+                                            b->plan.mblocks[mv], s));
   BATCH_TRY(b, rec(1));
   BATCH_TRY(b, launch_max_finalize_batch(pa, b->at<int32_t>(b->L.nb) + size_t(mv) * c, c, s));
   BATCH_TRY(b, rec(2));
@@ -453,7 +458,7 @@ int smc_batch_tune(smc_batch* b, int32_t reps, int32_t* choice_host) {
     for (int r = 0; r <= reps && e == cudaSuccess; ++r) {  // r == 0 warms up
       e = cudaEventRecord(e0, s);
       if (e == cudaSuccess)
-        e = launch_move_reweight_batch(pdry, gp, b->at<int4>(b->L.mmap[v]), int(b->plan.mmap[v].size()), s);
+        e = launch_move_reweight_classes(pdry, gp, b->at<int4>(b->L.mmap[v]), b->plan.mblocks[v], s);
       if (e == cudaSuccess) e = cudaEventRecord(e1, s);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms = 0.0f;
