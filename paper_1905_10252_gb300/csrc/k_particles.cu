@@ -17,6 +17,7 @@
 // paper's definitions, so its results are reproducible bit for bit.
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 
 #include "particle_bodies.cuh"
 #include "smc_internal.cuh"
@@ -590,13 +591,17 @@ __device__ __forceinline__ void move_reweight_body(const ParticleArgs& a, const 
   const int nvalid = d;
   const bool vec = ((d & 3) == 0) && (nvalid >= DPL);
   const BmStep bs = bm_step(float(a.step));
-  // Warp tiles of kEstTile consecutive particles (kEstChunks chunks of 32,
-  // lane l takes particle 32 r + l of chunk r), tile j to warp j mod W.  The
-  // loop bound is warp-uniform; lanes past the end are predicated.
-  constexpr int kChunks = kEstTile / 32;
+  // Warp tiles of kTile consecutive particles (kChunks chunks of 32, lane l
+  // takes particle 32 r + l of chunk r), tile j to warp j mod W.  The loop
+  // bound is warp-uniform; lanes past the end are predicated.  With the eq. (7)
+  // records a tile is a record's 256 particles; without them one chunk, so
+  // that few particles spread over all warps (N = 20011, D = 32: 79 warps with
+  // 8 chunks each took 17.5 us, 626 with one 6.6; N = 2^20 85 -> 74 us).  (Two
+  // chunks in a batch, where the warps of all members fill the SMs.)
+  constexpr int kTile = EST ? kEstTile : (std::is_same_v<FS, FactorSmem> ? 64 : 32), kChunks = kTile / 32;
   const int64_t gw = (int64_t(blk) * blockDim.x + threadIdx.x) >> 5;
   const int64_t W = int64_t(nblk) * (blockDim.x >> 5);
-  const int64_t ntile = (a.n + kEstTile - 1) / kEstTile;
+  const int64_t ntile = (a.n + kTile - 1) / kTile;
   const int grp = threadIdx.x & 31;
   int64_t j = gw;
   int r = 0;
@@ -605,7 +610,7 @@ __device__ __forceinline__ void move_reweight_body(const ParticleArgs& a, const 
   double lwc = 0.0;
   float lpc = 0.0f;
   {
-    const int64_t i = j * kEstTile + grp;
+    const int64_t i = j * kTile + grp;
     int64_t si = i;
     if constexpr (GATHER) {
       if (gat && j < ntile) {
@@ -627,7 +632,7 @@ __device__ __forceinline__ void move_reweight_body(const ParticleArgs& a, const 
   }
   bool first = true;
   while (j < ntile) {
-    const int64_t i = j * kEstTile + r * 32 + grp;
+    const int64_t i = j * kTile + r * 32 + grp;
     const bool valid = i < a.n;
     if (!PF && !first) {  // (the prologue loaded the first)
       if (valid && nvalid > 0) load_seg<DPL>(x + i * d + c0, vec, nvalid, xo);
@@ -640,7 +645,7 @@ __device__ __forceinline__ void move_reweight_body(const ParticleArgs& a, const 
     // the next particle: next chunk of this tile, or the first of the next
     const int rn = r + 1 == kChunks ? 0 : r + 1;
     const int64_t jn = r + 1 == kChunks ? j + W : j;
-    const int64_t inx = jn * kEstTile + rn * 32 + grp;
+    const int64_t inx = jn * kTile + rn * 32 + grp;
     const bool vn = jn < ntile && inx < a.n;
     constexpr int kPF = PF ? DPL : 1;
     float xn[kPF];
