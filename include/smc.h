@@ -173,7 +173,8 @@ int smc_redistribute(smc_sampler* h, const int32_t* ncopies_dev);
  * estimate, N_eff, and resample + redistribute + reset when N_eff < N*,
  * with no host synchronisation between iterations (the decision stays on the
  * device; the launches of an iteration are replayed from a CUDA graph).  An
- * FP64 sampler with N <= 2048 (Gaussian or Student-t target) runs the K
+ * FP64 sampler with N <= 256 (Gaussian or Student-t target) that does not
+ * resample in every iteration runs the K
  * iterations in one cooperative launch instead, with the same per-stage
  * arithmetic (bit-identical results); if its grid cannot be resident it uses
  * the graph. 

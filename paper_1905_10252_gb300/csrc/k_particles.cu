@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kPThreads) k_init(ParticleArgs a) {
       double q = 0.0;
 #pragma unroll
       for (int c = 0; c < DMAX; ++c) {
-        xr[c] = c < a.d ? __dmul_rn(a.init_scale, z[c]) : 0.0;
+        xr[c] = c < a.d ? __dmul_rn(2.0 * a.init_scale, z[c]) : 0.0;  // (z: half normals)
         if (c < a.d) q = __fma_rn(xr[c], xr[c], q);
       }
       const double lpi = (a.flags & PA_INIT_SKIP_LOGPI) ? 0.0 : eval_logpi<T, DMAX>(xr, a.d, a.kind, ts, nu, a.tg);
@@ -447,7 +447,7 @@ __device__ __forceinline__ void warp_write_est(float em, double R, float (&v)[DM
 // Algorithm 5 as a gather, for the 256 particles of move tile jt: row k of
 // the resampled set is row src(k) = the last run start at or before k
 // (rs[off_i] = i for every survivor i, -1 elsewhere).  tile_src holds src at
-// the first row of each 2048-row copy tile; run starts between that row and
+// the first row of each kRTile output rows; run starts between that row and
 // the move tile's first row are found by a backward search 32 rows at a time
 // (in all but heavily duplicated regions the 32 rows just before hold one).
 //

@@ -1796,18 +1796,18 @@ __global__ void __launch_bounds__(kRThreads) k_redistribute(RedistArgs a) {
 }
 
 // ---------------------------------------------------------------- one-tile samplers
-// A fused small sampler (N <= kSmallTile) that also returns the covariance
+// A fused small sampler that also returns the covariance
 // ends its last iteration with redistribute and commit as one kernel.
 template <typename V, int CPR>
 __global__ void __launch_bounds__(kRThreads) k_redistribute_commit(RedistArgs a, int d, int force_flip, int recycle) {
-  __shared__ RedistSmemT<kSmallTile> sm;
-  redistribute_body<V, CPR, 8, false, kSmallTile>(a, 0, sm);
+  __shared__ RedistSmemT<kRTile> sm;
+  redistribute_body<V, CPR, 8, false, kRTile>(a, 0, sm);
   __syncthreads();
   if (threadIdx.x < 32) commit_warp(a.st, d, force_flip, recycle);
 }
 
 // ---------------------------------------------------------------- fused small-sampler iterations
-// FP64 samplers of one quantise block and kSmallTile rows (N <= 2048): k
+// FP64 samplers of at most kSmallIter particles (see small_iter_fits): k
 // iterations of Algorithm 2 in one cooperative launch.  Every block runs its
 // share of the move + reweight with the particle-to-thread map of the
 // separate move launch (move_threads per block own particles); then block 0
@@ -1877,7 +1877,7 @@ union SmallIterSmem {
   TargetSmem<double> ts;
   QuantReduceSmem q;
   ScanSmem sc;
-  RedistSmemT<kSmallTile> r;
+  RedistSmemT<kRTile> r;
 };
 
 template <int DMAX, typename V>
@@ -1885,7 +1885,7 @@ __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
   __shared__ SmallIterSmem sm;
   TargetSmem<double>& ts = sm.ts;
   QuantReduceSmem& qsm = sm.q;
-  RedistSmemT<kSmallTile>& rsm = sm.r;
+  RedistSmemT<kRTile>& rsm = sm.r;
   DevState* st = s.a.st;
   unsigned long long* const bar = s.bar;
   unsigned long long nbar = 0;
@@ -1902,13 +1902,10 @@ __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
       __syncthreads();
       quant_finalize_body(s.q, 0);
       __syncthreads();
-      if (s.a.n <= kQThreads * 4)
-        quant_scan_body<4>(s.q, 0, s.q.cbase[0], sm.sc);
-      else
-        quant_scan_body<8>(s.q, 0, s.q.cbase[0], sm.sc);
+      quant_scan_body<1>(s.q, 0, s.q.cbase[0], sm.sc);
       if (!(s.stop_last && it + 1 == s.k)) {
         __syncthreads();
-        redistribute_body<V, 0, 8, true, kSmallTile>(s.r, 0, rsm);
+        redistribute_body<V, 0, 8, true, kRTile>(s.r, 0, rsm);
         __syncthreads();
         if (threadIdx.x < 32) commit_warp(st, s.d, 0, 1);
       }
@@ -1917,7 +1914,15 @@ __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
   }
 }
 
-bool small_iter_fits(int64_t n, int dtype) { return dtype == SMC_F64 && n <= kSmallTile && n <= kQTile; }
+// Up to kSmallIter particles, unless every iteration resamples.  Measured per
+// iteration (fused, separate kernels): N = 64, D = 1 21.9, 24.3 us; N = 256, D = 1
+// 22.4, 23.9; N = 256, D = 4 29.2, 28.9; N = 1024, D = 4 32.0, 30.4; N = 2048, D = 32
+// 160, 111; and with a copy in every iteration N = 64, D = 1 26.7, 25.9, N = 256, D = 4
+// 32.2, 30.0 (block 0's stages one after another against many blocks each).
+static_assert(kSmallIter <= kRTile && kSmallIter <= kQThreads, "one copy tile, one scan item per thread");
+bool small_iter_fits(int64_t n, int dtype, int mode) {
+  return dtype == SMC_F64 && n <= kSmallIter && mode != SMC_RESAMPLE_ALWAYS;
+}
 
 template <int DMAX>
 static cudaError_t iterate_small_d(const SmallIterArgs& s, int blocks, cudaStream_t st) {
@@ -1929,7 +1934,7 @@ static cudaError_t iterate_small_d(const SmallIterArgs& s, int blocks, cudaStrea
 }
 
 cudaError_t launch_iterate_small(const SmallIterArgs& s, int move_blocks, cudaStream_t st) {
-  if (!small_iter_fits(s.a.n, s.a.dtype) || s.k < 1 || move_blocks < 1 || s.move_threads < 1 ||
+  if (!small_iter_fits(s.a.n, s.a.dtype, s.q.mode) || s.k < 1 || move_blocks < 1 || s.move_threads < 1 ||
       s.move_threads > kQThreads || s.d < 1 || s.d > kMaxD || s.r.row_bytes % 8 != 0)
     return cudaErrorInvalidValue;
   if (s.d <= 4) return iterate_small_d<4>(s, move_blocks, st);
@@ -2187,7 +2192,7 @@ cudaError_t launch_redistribute(const RedistArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_redistribute_commit(const RedistArgs& a, int d, int force_flip, int recycle, cudaStream_t s) {
-  if (a.n > kSmallTile) return cudaErrorInvalidValue;
+  if (a.n > kRTile) return cudaErrorInvalidValue;
   const int rb = a.row_bytes;
   if (rb % 16 == 0) {
     switch (rb / 16) {

@@ -13,10 +13,24 @@
 namespace smc {
 
 // ---------------------------------------------------------------- log targets
+// a / b, correctly rounded, from y = RN(1 / b): two residual steps bring q
+// within an ulp, and with a correctly rounded reciprocal the last one rounds
+// correctly (Markstein, IBM J. Res. Dev. 34, 1990).  Five FP64
+// operations; operands near the ends of the exponent range, zeros, infinities
+// and NaN divide as usual.
+__device__ __forceinline__ double div_by_known(double a, double b, double y) {
+  const double q0 = __dmul_rn(a, y);
+  const unsigned ea = (unsigned(__double2hiint(a)) >> 20) & 0x7ff, eq = (unsigned(__double2hiint(q0)) >> 20) & 0x7ff;
+  if (ea - 200u > 1600u || eq - 200u > 1600u) return __ddiv_rn(a, b);
+  const double q1 = __fma_rn(__fma_rn(-b, q0, a), y, q0);
+  return __fma_rn(__fma_rn(-b, q1, a), y, q1);
+}
+
 // Gaussian, FP64: forward substitution z = L^-1 (x - mu), log pi = -1/2 |z|^2.
+// rd: the reciprocals of L's diagonal (the diagonal of L^-1), correctly rounded.
 template <int DMAX>
 __device__ __forceinline__ double logpi_gauss(const double (&x)[DMAX], int d, const double* __restrict__ L,
-                                              const double* __restrict__ mu) {
+                                              const double* __restrict__ mu, const double* __restrict__ rd) {
   double z[DMAX];
   double q = 0.0;
 #pragma unroll
@@ -25,7 +39,7 @@ __device__ __forceinline__ double logpi_gauss(const double (&x)[DMAX], int d, co
       double acc = __dsub_rn(x[r], mu[r]);
 #pragma unroll
       for (int c = 0; c < r; ++c) acc = __fma_rn(-L[r * kMaxD + c], z[c], acc);
-      z[r] = __ddiv_rn(acc, L[r * kMaxD + r]);
+      z[r] = div_by_known(acc, L[r * kMaxD + r], rd[r]);
       q = __fma_rn(z[r], z[r], q);
     }
   }
@@ -35,7 +49,7 @@ __device__ __forceinline__ double logpi_gauss(const double (&x)[DMAX], int d, co
 // Gaussian, FP32: y = P (x - mu) with the precomputed inverse factor.
 template <int DMAX>
 __device__ __forceinline__ float logpi_gauss(const float (&x)[DMAX], int d, const float* __restrict__ P,
-                                             const float* __restrict__ mu) {
+                                             const float* __restrict__ mu, const float* __restrict__) {
   float dv[DMAX];
 #pragma unroll
   for (int c = 0; c < DMAX; ++c) dv[c] = c < d ? x[c] - mu[c] : 0.0f;
@@ -162,6 +176,7 @@ template <typename T>
 struct TargetSmem {
   T mu[kMaxD];
   T F[kMaxD * kMaxD];  // L (FP64 path) or P (FP32 path)
+  T rd[kMaxD];         // FP64: 1 / L[r][r]
 };
 
 template <typename T>
@@ -169,8 +184,11 @@ __device__ __forceinline__ void load_target(const TargetDev* __restrict__ tg, in
 template <>
 __device__ __forceinline__ void load_target<double>(const TargetDev* __restrict__ tg, int d,
                                                     TargetSmem<double>& s) {
-  for (int i = threadIdx.x; i < kMaxD * kMaxD; i += blockDim.x) s.F[i] = tg->L[i];
-  for (int i = threadIdx.x; i < kMaxD; i += blockDim.x) s.mu[i] = tg->mu[i];
+  for (int i = threadIdx.x; i < d * kMaxD; i += blockDim.x) s.F[i] = tg->L[i];
+  for (int i = threadIdx.x; i < kMaxD; i += blockDim.x) {
+    s.mu[i] = tg->mu[i];
+    s.rd[i] = tg->P[i * kMaxD + i];
+  }
   __syncthreads();
 }
 template <>
@@ -185,7 +203,7 @@ __device__ __forceinline__ T eval_logpi(const T (&x)[DMAX], int d, int kind, con
                                         const TargetDev* __restrict__ tg) {
   if (kind == SMC_STUDENT_T) return logpi_student(x[0], ts.mu[0], nu);
   if (kind == SMC_LOGISTIC) return logpi_logistic<DMAX>(x, d, tg);
-  return logpi_gauss<DMAX>(x, d, ts.F, ts.mu);
+  return logpi_gauss<DMAX>(x, d, ts.F, ts.mu, ts.rd);
 }
 
 // ---------------------------------------------------------------- move + reweight
@@ -217,7 +235,7 @@ __device__ __forceinline__ void move_reweight_generic_body(const ParticleArgs& a
         normals_f64<DMAX>(a.seed, t, kPurposeMove, uint64_t(i), a.d, z);
 #pragma unroll
         for (int c = 0; c < DMAX; ++c)
-          if (c < a.d) xr[c] = __fma_rn(a.step, z[c], xr[c]);
+          if (c < a.d) xr[c] = __fma_rn(2.0 * a.step, z[c], xr[c]);  // (z: half normals)
       } else {
         float z[DMAX];
         normals_f32<DMAX>(a.seed, t, kPurposeMove, uint64_t(i), a.d, z);

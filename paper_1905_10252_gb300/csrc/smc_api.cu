@@ -448,12 +448,16 @@ int smc_init(smc_sampler** out, const smc_config* cfg, void* x_dev, void* x_alt_
   h->tile_src = reinterpret_cast<int32_t*>(h->ws + L.tile_src);
   // particle kernels: 256-thread blocks, at most 8 per SM (grid-stride);
   // samplers of fewer than 256 particles per SM use one-warp blocks so that
-  // their work (FP64 in particular) spreads over the SMs
+  // their work (FP64 in particular) spreads over the SMs.  FP64 samplers:
+  // always one-warp blocks, 16 per SM: their time is the FP64 pipe's, so every
+  // SM should get the same share (five iterations at N = 2^18, D = 8: 1144 us;
+  // with 1024 blocks of 256 threads 1195, with a block per 64 particles 1220).
   {
     const int64_t units = h->n * lanes_per_particle(h->dtype, h->d);
     const int64_t sms = sm_count();
-    h->threads_p = units < int64_t(kPThreads) * sms ? 32 : kPThreads;
-    h->grid_p = int(std::min<int64_t>(div_up(units, h->threads_p), sms * 8));
+    const bool f64 = h->dtype == SMC_F64;
+    h->threads_p = f64 || units < int64_t(kPThreads) * sms ? 32 : kPThreads;
+    h->grid_p = int(std::min<int64_t>(div_up(units, h->threads_p), sms * (f64 ? 16 : 8)));
     if (h->grid_p > kMaxPartBlocks) h->grid_p = kMaxPartBlocks;
   }
   h->lg_tc = cfg->target == SMC_LOGISTIC && cfg->dtype == SMC_F32 && !(cfg->flags & SMC_FLAG_LOGISTIC_CUDA_CORES);
@@ -497,7 +501,7 @@ int smc_init(smc_sampler** out, const smc_config* cfg, void* x_dev, void* x_alt_
   h->defer = (cfg->flags & SMC_FLAG_DEFER_REDISTRIBUTE) && est_in_move(h) && h->L.qblocks > 1;
   // small FP64 samplers (generic move kernel, one quantise block, one block's
   // copy): smc_step fuses their iterations into one cooperative launch
-  h->small_iter = small_iter_fits(h->n, h->dtype) && cfg->target != SMC_LOGISTIC && !h->defer && h->L.qblocks == 1;
+  h->small_iter = small_iter_fits(h->n, h->dtype, cfg->resample_mode) && cfg->target != SMC_LOGISTIC && !h->defer;
   if (e != cudaSuccess) {
     int r = cuda_fail(nullptr, e, "smc_init launch");
     delete h;

@@ -31,7 +31,7 @@ constexpr int kQSplit = 8;            // blocks that share a tile in the passes 
 constexpr int kQSplitTiles = 76;       // ... of at most this many tiles
 constexpr int kRTile = 512;            // output rows per source entry (tile_src, stamps) of the redistribute copy
 constexpr int kCopyTile = 1024;        // output rows per block of the copy of large samplers and of batches
-constexpr int kSmallTile = 2048;      // ... of the one-block copy of a fused small sampler
+constexpr int kSmallIter = 256;       // particles of a sampler whose iterations are one launch, at most
 constexpr int kRThreads = 256;
 constexpr int kPThreads = 256;        // particle kernels (init / move / reweight)
 constexpr int kFinThreads = 1024;     // single-block finalisers
@@ -188,16 +188,30 @@ __device__ __forceinline__ P4 stream_block(uint64_t seed, uint64_t t, uint32_t p
 __device__ __forceinline__ double ln2_hi() { return __longlong_as_double(0x3FE62E42FEE00000ll); }
 __device__ __forceinline__ double ln2_lo() { return __longlong_as_double(0x3DEA39EF35793C76ll); }
 
-// log(u), u finite, normal, > 0: u = 2^e m, m in [sqrt(1/2), sqrt(2)),
-// log m = 2 atanh(s), s = (m-1)/(m+1), series to s^22.
-__device__ __forceinline__ double det_log(double u) {
-  const long long b = __double_as_longlong(u);
-  int e = int((b >> 52) & 0x7ff) - 1023;
-  double m = __longlong_as_double((b & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
-  if (m > __longlong_as_double(0x3FF6A09E667F3BCDll)) {
-    m = __dmul_rn(m, 0.5);
+// An FP64 instruction takes an SM 16 cycles per warp (an integer one a quarter
+// to half of one), so what is exact by construction is done on the bits:
+// conversions of integers, scalings by powers of two, comparisons.  The FP64
+// operations that remain are those of the definition, in its order and with
+// its roundings (a power of two taken out of a chain changes no rounding).
+// (With the target's divisions by known divisors, five iterations at N = 2^18, D = 8:
+// 1318 us with them as FP64 instructions, 1195 without.)
+
+// The double of an integer 0 <= v <= 2^53.
+__device__ __forceinline__ double exact_double(uint64_t v) {
+  const int lz = __clzll((long long)v);
+  const uint64_t bits = (uint64_t(1086 - lz) << 52) + (((v << lz) << 1) >> 12);
+  return __longlong_as_double((long long)(v ? bits : 0ull));
+}
+
+// log(m 2^e) / 2 for a significand given by its bits (1 <= m < 2): m brought to
+// [sqrt(1/2), sqrt(2)), log m = 2 atanh(s), s = (m-1)/(m+1), series to s^22.
+// Half the logarithm: the factor 2 of atanh is left out, and ln 2 halved.
+__device__ __forceinline__ double det_log_half(uint64_t mbits, int e) {
+  if (mbits > 0x3FF6A09E667F3BCDull) {
+    mbits -= 1ull << 52;  // m / 2
     e += 1;
   }
+  const double m = __longlong_as_double((long long)mbits);
   const double s = __ddiv_rn(__dsub_rn(m, 1.0), __dadd_rn(m, 1.0));
   const double s2 = __dmul_rn(s, s);
   double p = 1.0 / 23.0;
@@ -212,9 +226,17 @@ __device__ __forceinline__ double det_log(double u) {
   p = __fma_rn(p, s2, 1.0 / 5.0);
   p = __fma_rn(p, s2, 1.0 / 3.0);
   p = __fma_rn(p, s2, 1.0);
-  const double logm = __dmul_rn(__dmul_rn(2.0, s), p);
-  const double de = double(e);
-  return __fma_rn(de, ln2_hi(), __fma_rn(de, ln2_lo(), logm));
+  const double h = __dmul_rn(s, p);
+  const unsigned n = unsigned(e < 0 ? -e : e);  // below 2^11: the double of e in the high word
+  const int lz = __clz(int(n));
+  const double de = __hiloint2double(n ? int((e < 0 ? 0x80000000u : 0u) | (unsigned(1054 - lz) << 20) | ((n << lz) << 1 >> 12)) : 0, 0);
+  return __fma_rn(de, 0.5 * ln2_hi(), __fma_rn(de, 0.5 * ln2_lo(), h));
+}
+
+// log(u), u finite, normal, > 0.
+__device__ __forceinline__ double det_log(double u) {
+  const uint64_t b = (uint64_t)__double_as_longlong(u);
+  return __dmul_rn(2.0, det_log_half((b & 0x000FFFFFFFFFFFFFull) | 0x3FF0000000000000ull, int((b >> 52) & 0x7ff) - 1023));
 }
 
 // sin and cos of 2 pi v 2^-53 (0 <= v < 2^53): exact quarter-turn reduction on
@@ -222,8 +244,9 @@ __device__ __forceinline__ double det_log(double u) {
 __device__ __forceinline__ void det_sincos2pi(uint64_t v, double* s_out, double* c_out) {
   const uint64_t q = (v + (1ull << 50)) >> 51;
   const long long vr = (long long)v - (long long)(q << 51);
-  const double x = __dmul_rn(double(vr), 0x1p-53);
-  const double t = __dmul_rn(x, __longlong_as_double(0x401921FB54442D18ll));  // 2 pi
+  const double xm = exact_double(uint64_t(vr < 0 ? -vr : vr));  // |x| 2^53
+  const double x = __hiloint2double(__double2hiint(xm) | (vr < 0 ? int(0x80000000) : 0), __double2loint(xm));
+  const double t = __dmul_rn(x, __longlong_as_double(0x3CC921FB54442D18ll));  // 2 pi 2^-53
   const double t2 = __dmul_rn(t, t);
   double ps = -1.0 / 121645100408832000.0;
   ps = __fma_rn(ps, t2, 1.0 / 355687428096000.0);
@@ -254,9 +277,10 @@ __device__ __forceinline__ void det_sincos2pi(uint64_t v, double* s_out, double*
   }
 }
 
-// D standard normals (FP64 path): pair p uses block p, whose four 32-bit words
-// make the 64-bit words (w0 w1) and (w2 w3); their top 53 bits are a and b;
-// u1 = 1 - a, r = sqrt(-2 log u1), (z0, z1) = r (cos, sin)(2 pi b).
+// D standard normals (FP64 path), each divided by 2: pair p uses block p, whose
+// four 32-bit words make the 64-bit words (w0 w1) and (w2 w3); their top 53
+// bits are a and b; u1 = 1 - a, r = sqrt(-2 log u1), (z0, z1) = r (cos,
+// sin)(2 pi b).  Here r / 2 = sqrt(-(log u1) / 2); the callers' scale is doubled.
 template <int DMAX>
 __device__ __forceinline__ void normals_f64(uint64_t seed, uint64_t t, uint32_t purpose, uint64_t i, int d,
                                             double (&z)[DMAX]) {
@@ -266,8 +290,10 @@ __device__ __forceinline__ void normals_f64(uint64_t seed, uint64_t t, uint32_t 
       const P4 w = stream_block(seed, t, purpose, i, uint32_t(p));
       const uint64_t va = ((uint64_t(w.v[0]) << 32) | w.v[1]) >> 11;
       const uint64_t vb = ((uint64_t(w.v[2]) << 32) | w.v[3]) >> 11;
-      const double u1 = __dmul_rn(double((1ull << 53) - va), 0x1p-53);
-      const double r = __dsqrt_rn(__dmul_rn(-2.0, det_log(u1)));
+      // u1 = v 2^-53 by its significand and exponent
+      const uint64_t v = (1ull << 53) - va;
+      const int lz = __clzll((long long)v);
+      const double r = __dsqrt_rn(-det_log_half(0x3FF0000000000000ull | (((v << lz) << 1) >> 12), 10 - lz));
       double sn, cs;
       det_sincos2pi(vb, &sn, &cs);
       z[2 * p] = __dmul_rn(r, cs);

@@ -263,11 +263,11 @@ cudaError_t launch_iter_scan(const QuantArgs& a, cudaStream_t s);
 bool nc_small(int64_t n);  // the scan writes every run start itself: no stamps at this size
 cudaError_t launch_nc(const NcScanArgs& a, cudaStream_t s);  // exclusive scan of ncopies: run starts, tile sources
 cudaError_t launch_redistribute(const RedistArgs& a, cudaStream_t s);
-// fused small samplers (N <= kSmallTile): redistribute + commit as one launch
+// fused small samplers: redistribute + commit as one launch
 cudaError_t launch_redistribute_commit(const RedistArgs& a, int d, int force_flip, int recycle, cudaStream_t s);
 
-// k iterations of an FP64 sampler of one quantise block and one copy tile
-// (N <= 2048) in one cooperative launch of move_blocks blocks (see
+// k iterations of a small FP64 sampler (small_iter_fits)
+// in one cooperative launch of move_blocks blocks (see
 // k_iterate_small).  bar: the grid barrier's zeroed 64-bit count.  stop_last: the
 // last iteration ends after its scan (its copy and commit follow as separate
 // launches, after the covariance).
@@ -283,7 +283,7 @@ struct SmallIterArgs {
   int32_t stall;  // test hook (SMC_FLAG_TEST_STALL_BARRIER): the barrier waits for one block more than the grid
   int32_t pad;
 };
-bool small_iter_fits(int64_t n, int dtype);
+bool small_iter_fits(int64_t n, int dtype, int mode);
 cudaError_t launch_iterate_small(const SmallIterArgs& s, int move_blocks, cudaStream_t st);
 int nearly_sort_tiles(int64_t n);
 cudaError_t launch_nearly_sort(const NearlySortArgs& a, cudaStream_t s);
