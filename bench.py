@@ -556,9 +556,9 @@ def run_iteration(args):
     redist = None
     if rank == 0 and ws == 1 and not args.no_redistribute:
         redist = redistribute_summary(1 << 24, 16, ["s0.5", "s2", "s8", "onehot"], 0, 20, peak)
-    # one step set-up per smc_step call, then per iteration: begin, move +
-    # reweight, max, quantise reduce / finalise, scan, (redistribute,) commit
-    launches_per_step = 7 if gather else 8
+    # one step set-up per smc_step call, then per iteration: move + reweight,
+    # quantise reduce, finalise, scan with the statistics (, redistribute)
+    launches_per_step = 4 if gather else 5
     if rank == 0:
         line = {
             "metric": METRIC, "value": value, "unit": METRIC, "n_gpus": ws, "steps": K, "warmup": W,
@@ -569,7 +569,7 @@ def run_iteration(args):
                        "l2": "inputs larger than L2 (particle state %.2f GB per buffer)" % (n * d * 4 / 1e9),
                        "redistribute": ("gathered by the next iteration's move (SMC_FLAG_DEFER_REDISTRIBUTE)"
                                         if gather else "copy kernel at the end of the iteration")},
-            "entry_point": f"smc_step (one call, {K} iterations replayed from the sampler's CUDA graph)",
+            "entry_point": f"smc_step (one call, {K} iterations, replayed from the sampler's CUDA graphs)",
             "roofline": roof(dominant) if dominant in byt else roof("move_reweight"),
             "dominant_kernel": dominant,
             "profile_pass": {"entry_point": "smc_step_profile (direct launches, events between stages)",
@@ -785,7 +785,9 @@ def run_batch(args):
             "stage_roofline": {"move_reweight": roof("move_reweight", mv_bytes),
                                "quantise_reduce_estimate": roof("quantise_reduce_estimate", q_bytes)},
             "stages_ms": {k: round(v, 5) for k, v in stage_ms.items()},
-            "gpu_launches": 8 * K,
+            # begin, one move launch per width class, max, quantise reduce /
+            # finalise, scan, copy, commit
+            "gpu_launches": (7 + len({(d > 16) + (d > 8) + 3 * (d in (8, 16, 32)) for _, d in shapes})) * K,
             "clocks": clocks.summary(t_host0, t_host1),
         }
         print(json.dumps(line), flush=True)
@@ -857,7 +859,8 @@ def run_logistic(args):
     sm_mhz = clk.get("sm_mhz") or 2070.0
     lik_ms = stage_ms["move_reweight"]
     elems = float(n) * float(((m + 255) // 256) * 256)
-    mufu_peak = 152 * 16 * sm_mhz * 1e6 / 1.0625  # elements/s: one ex2 + 1/16 lg2 per element, 16 MUFU lanes / SM
+    # elements/s: one ex2 (32 lanes per SM and clock on this GPU) and 1/16 lg2 (16 lanes) per element
+    mufu_peak = 152 * sm_mhz * 1e6 / (1 / 32 + 1 / 256)
     tensor_flops = 3 * 2.0 * elems * 32
     meas = {}
     try:
@@ -877,14 +880,15 @@ def run_logistic(args):
             "roofline": {"bound": "alu", "achieved": round(elems / (lik_ms * 1e-3) / 1e9, 1),
                          "peak": round(mufu_peak / 1e9, 1), "unit": "Gelem/s",
                          "frac": round(elems / (lik_ms * 1e-3) / mufu_peak, 4), "traffic": None,
-                         "note": "move + likelihood stage; peak = MUFU rate at the sampled SM clock / 1.0625 ops "
-                                 "per element"},
+                         "note": "move + likelihood stage; peak = MUFU rate at the sampled SM clock: one ex2 at 32 "
+                                 "and 1/16 lg2 at 16 lanes per SM and clock per element"},
             "tensor": {"achieved_tflops": round(tensor_flops / (lik_ms * 1e-3) / 1e12, 1),
                        "peak_tflops": bf16_peak, "frac": round(tensor_flops / (lik_ms * 1e-3) / 1e12 / bf16_peak, 4)},
             "likelihood_ms": {"tensor_cores": round(lik_ms, 4), "cuda_cores_fp32": round(cc_ms, 4),
                               "speedup": round(cc_ms / lik_ms, 2)},
             "stages_ms": {k: round(v, 5) for k, v in stage_ms.items()},
-            "gpu_launches": 9 * K,
+            # move, likelihood, quantise reduce, finalise, scan, redistribute
+            "gpu_launches": 6 * K,
             "clocks": clk,
         }
         print(json.dumps(line), flush=True)
@@ -1011,9 +1015,7 @@ def run_c0(args):
     times, cold, errs = [], [], []
     for r in range(args.warmup + reps):
         # cold: a fresh sampler's first K iterations; warm: K more iterations
-        # of the same sampler (the steady cost of a resident job).  smc_step
-        # runs the K iterations of this FP64 sampler of 1024 particles in one
-        # cooperative launch (then the covariance and the last copy)
+        # of the same sampler (the steady cost of a resident job)
         S = native.Sampler(N, D, dtype=torch.float64, seed=r, mu=mu, sigma=Sigma, step=0.5, init_scale=2.0)
         torch.cuda.synchronize()
         e0, e1, e2 = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
@@ -1037,11 +1039,10 @@ def run_c0(args):
             "config": {"workload": "plain fp64 sampler N=1024 D=4 K=20 gauss, resample when N_eff < N/2",
                        "timing": f"median over {reps} runs (seeds) of K more iterations of a resident sampler "
                                  "(one smc_step call), CUDA events on its stream",
-                       "entry_point": "smc_step (K iterations in one cooperative launch, then the covariance "
-                                      "and the last copy + commit)"},
+                       "entry_point": "smc_step (K iterations of five kernels, the covariance in the last)"},
             "particle_iters_per_s": N * K / (us * 1e-6), "cold_us_first_call": float(np.median(cold)),
             "mean_abs_err_max_vs_closed_form": {"median": float(np.median(errs)), "max": float(np.max(errs))},
-            "gpu_launches": 5}), flush=True)  # step set-up, the fused iterations, covariance (2), copy + commit
+            "gpu_launches": 1 + 5 * K + 2}), flush=True)  # step set-up, the iterations, covariance (2)
 
 
 def main():

@@ -172,12 +172,13 @@ int smc_redistribute(smc_sampler* h, const int32_t* ncopies_dev);
 /* K iterations of Algorithm 2 (lines 3-10): move, reweight, normalise,
  * estimate, N_eff, and resample + redistribute + reset when N_eff < N*,
  * with no host synchronisation between iterations (the decision stays on the
- * device; the launches of an iteration are replayed from a CUDA graph).  An
+ * device; the launches are replayed from CUDA graphs once a sampler has run
+ * its first iterations by plain launches).  An
  * FP64 sampler with N <= 256 (Gaussian or Student-t target) that does not
  * resample in every iteration runs the K
  * iterations in one cooperative launch instead, with the same per-stage
  * arithmetic (bit-identical results); if its grid cannot be resident it uses
- * the graph. 
+ * separate launches.
  * mean_dev[D] receives f_K, cov_dev[D*D] (may be NULL) the final weighted
  * covariance, trace_dev (may be NULL) K smc_iter_stats records, and
  * fhat_dev[D] (may be NULL) the recycled estimate of eq. (6) over all
@@ -189,7 +190,8 @@ int smc_step(smc_sampler* h, int32_t k, double* mean_dev, double* cov_dev, smc_i
  * with events_host[0] (cudaEvent_t, created by the caller) recorded before it
  * and events_host[j] after stage j: 1 move + reweight, 2 max / mean finalise,
  * 3 quantise reduce, 4 quantise finalise, 5 systematic scan, 6 redistribute,
- * 7 commit.  n_events must be 8, or 0 to record nothing.  The iteration is
+ * 7 commit (the maximum, the mean and the commit are part of the kernels
+ * around them, so 2 and 7 follow at once).  n_events must be 8, or 0 to record nothing.  The iteration is
  * identical to one iteration of smc_step (mean_dev may be NULL). */
 int smc_step_profile(smc_sampler* h, double* mean_dev, void* const* events_host, int32_t n_events);
 
@@ -350,7 +352,8 @@ int smc_batch_create(smc_batch** out, smc_sampler* const* members, int32_t count
 /* k iterations for every member.  mean_dev / trace_dev / fhat_dev are NULL or
  * HOST arrays of count DEVICE pointers (entries may be NULL) with the meaning
  * smc_step gives its arguments of those names, per member.  Iterations are
- * replayed from a CUDA graph of one batched iteration (8 launches). */
+ * replayed from a CUDA graph of one batched iteration (one launch per stage,
+ * the move one per width class). */
 int smc_batch_step(smc_batch* b, int32_t k, double* const* mean_dev, smc_iter_stats* const* trace_dev,
                    double* const* fhat_dev);
 

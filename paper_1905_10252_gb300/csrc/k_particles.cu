@@ -867,8 +867,8 @@ __global__ void k_begin(DevState* st) {
   if (threadIdx.x == 0) st->t += 1;
 }
 
-__global__ void k_commit(DevState* st, int d, int force_flip, int recycle, int defer) {
-  if (threadIdx.x < 32) commit_warp(st, d, force_flip, recycle, defer);
+__global__ void k_commit(DevState* st, int d, int force_flip, int recycle) {
+  if (threadIdx.x < 32) commit_warp(st, d, force_flip, recycle);
 }
 
 __global__ void k_settle(DevState* st) {
@@ -1089,8 +1089,8 @@ cudaError_t launch_begin(DevState* st, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_commit(DevState* st, int d, int force_flip, int recycle, cudaStream_t s, int defer) {
-  k_commit<<<1, 32, 0, s>>>(st, d, force_flip, recycle, defer);
+cudaError_t launch_commit(DevState* st, int d, int force_flip, int recycle, cudaStream_t s) {
+  k_commit<<<1, 32, 0, s>>>(st, d, force_flip, recycle);
   return cudaGetLastError();
 }
 

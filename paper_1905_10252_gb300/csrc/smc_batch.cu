@@ -174,7 +174,8 @@ int bfail(smc_batch* b, int code, const std::string& msg) {
     if (_e != cudaSuccess) return bfail((b), SMC_ECUDA, std::string(#expr) + ": " + cudaGetErrorString(_e)); \
   } while (0)
 
-// One iteration of Algorithm 2 (lines 3-10) for every member: 8 launches.
+// One iteration of Algorithm 2 (lines 3-10) for every member: one launch per
+// stage, the move one per width class.
 cudaError_t launch_batch_iteration(const smc_batch* b) {
   const int c = b->count, mv = b->move_v;
   cudaStream_t s = b->stream;

@@ -521,12 +521,10 @@ __device__ __forceinline__ uint64_t quotient_2p64(uint64_t n, uint64_t S) {
 // (0 after a reset), and the recycling sums of eq. (6) take f_t with weight
 // c_t -- one column per lane, each with explicitly rounded FP64 operations
 // (the same bits whichever kernel runs it).
-// defer: a resampled iteration leaves its rows in place and marks them
-// pending instead of swapping (the next move gathers them).
 // Every field the commit reads is loaded before its first store (one round
 // trip to memory instead of a chain of them; the values are those the
 // original order reads, as no field is read after the commit writes it).
-__device__ __forceinline__ void commit_warp(DevState* st, int d, int force_flip, int recycle, int defer = 0) {
+__device__ __forceinline__ void commit_warp(DevState* st, int d, int force_flip, int recycle) {
   const int lane = threadIdx.x & 31;
   const int err = st->err, flag = st->flag, cur = st->cur;
   const double lc = st->logc, rmax = st->rc_max, rden = st->rc_den, lse = st->lse;
@@ -542,8 +540,7 @@ __device__ __forceinline__ void commit_warp(DevState* st, int d, int force_flip,
     rnum[j] = c < d ? st->rc_num[c] : 0.0;
     mc[j] = c < d ? st->mean[c] : 0.0;
   }
-  const bool pend = defer && flag && !err;
-  const bool flip = force_flip || (flag && !err && !defer);
+  const bool flip = force_flip || (flag && !err);
   double M = 0.0, den = 0.0;
   if (recycle && !err) {
     M = fmax(rmax, lc);
@@ -574,10 +571,9 @@ __device__ __forceinline__ void commit_warp(DevState* st, int d, int force_flip,
     }
   }
   if (flip) st->cur = cur ^ 1;
-  st->pending = pend ? 1 : 0;
-  st->lse_prev = (flip || pend) ? 0.0 : lse;
+  st->lse_prev = flip ? 0.0 : lse;
   // a resampled iteration leaves every log w at reset_logw
-  st->w_uniform = ((flip || pend) && !err) ? 1 : 0;
+  st->w_uniform = (flip && !err) ? 1 : 0;
 }
 
 }  // namespace smc

@@ -208,7 +208,7 @@ cudaError_t launch_max_finalize(const double* part, int nb, DevState* st, cudaSt
 // eq. (7) covariance (k_moments.cu): grid blocks write covpart[grid][D(D+1)/2], then a fixed-order sum
 cudaError_t launch_cov(const ParticleArgs& a, double* cov, double* covpart, int grid, cudaStream_t s);
 cudaError_t launch_begin(DevState* st, cudaStream_t s);
-cudaError_t launch_commit(DevState* st, int d, int force_flip, int recycle, cudaStream_t s, int defer = 0);
+cudaError_t launch_commit(DevState* st, int d, int force_flip, int recycle, cudaStream_t s);
 // Ends a pending (deferred) redistribution after its copy: the copied rows'
 // buffer becomes current.
 cudaError_t launch_settle(DevState* st, cudaStream_t s);
