@@ -205,7 +205,15 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
     if constexpr (kF32) {
       float h = 0.0f, l = 0.0f;
       int E = -(1 << 20);
-      if (lw != -INFINITY) exp_split(m - lw, s_T, h, l, E);
+      if (lw != -INFINITY) {
+        const double a_i = m - lw;
+        if (a_i > -INFINITY) {
+          exp_split(a_i, s_T, h, l, E);
+        } else {  // e^{inf} or NaN (log w is NaN or +inf, which the reweight reports): what it makes of the sums
+          h = a_i == -INFINITY ? INFINITY : NAN;
+          E = 0;
+        }
+      }
       const int em = __reduce_max_sync(0xffffffffu, E);
       if ((tid & 31) == 0) atomicMax(&s_emax[turn], em);
       __syncthreads();

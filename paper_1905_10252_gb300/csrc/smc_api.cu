@@ -419,6 +419,8 @@ int smc_init(smc_sampler** out, const smc_config* cfg, void* x_dev, void* x_alt_
   const Layout L = layout_for(cfg->n, cfg->d, logistic_rows(cfg), wants_two_rs(cfg));
   if (workspace_bytes < L.total) return fail(nullptr, SMC_ENOMEM, "workspace too small");
   cudaError_t e = upload_expfx_table();
+  const uint64_t* table = nullptr;  // (looked up here once, not first under a caller's stream capture)
+  if (e == cudaSuccess) e = expfx_table(&table);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "upload_expfx_table");
 
   smc_sampler* h = new (std::nothrow) smc_sampler();

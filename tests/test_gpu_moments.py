@@ -97,3 +97,13 @@ def test_covariance_of_far_apart_weights(nat, gap):
     mean2, cov = S.estimate(cov=True)
     assert torch.equal(mean, mean2)
     _check(nat, S, mean, cov, torch.float32)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_nan_weight_reaches_the_covariance(nat, dtype):
+    S = _sampler(nat, 700, 5, dtype)
+    S.move()
+    S.reweight()
+    S.logw[123] = float("nan")
+    _, cov = S.estimate(cov=True)
+    assert bool(torch.isnan(cov).all())
