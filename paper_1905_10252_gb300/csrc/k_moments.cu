@@ -16,10 +16,9 @@
 // division per row) took 4.59 ms at N = 2^20, D = 32.  FP32 samplers
 // therefore keep u and every sum as an unevaluated pair of FP32 values
 // (error-free product by FMA, Knuth's two-sum: Dekker 1971; Knuth, TAOCP 2,
-// 4.2.2), 11 FP32
-// operations per pair, and the weight comes from the
-// integer exponential of the quantise pass with its exponent kept apart, so
-// that a weight far below the largest keeps its relative precision.  The sums
+// 4.2.2), 11 FP32 operations per pair, and the weight comes from the integer
+// exponential of the quantise pass with its exponent kept apart, so that a
+// weight far below the largest keeps its relative precision.  The sums
 // carry about 2^-45 relative error, far below the 2^-25 of rounding a row's
 // difference to FP32 (the row precision), and no FP64 operation is left on
 // the per-pair path.  FP64 samplers use FP64 FMAs, one per pair.

@@ -19,6 +19,7 @@
 //    vector loads/stores.  Every tile does the same bounded work whatever the
 //    weights.  Replaces the paper's MPI nearly-sort and rotational shifts
 //    (Sec. 4) with O(1) passes over the data.
+#include <atomic>
 #include <cmath>
 
 #include "particle_bodies.cuh"
@@ -77,19 +78,18 @@ cudaError_t upload_expfx_table() {
 // The device copy of the table on the current device, for the kernels of
 // other translation units.
 cudaError_t expfx_table(const uint64_t** out) {
-  static const uint64_t* at[64] = {nullptr};
+  static std::atomic<const uint64_t*> at[64];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64 && at[dev]) {
-    *out = at[dev];
-    return cudaSuccess;
-  }
+  const bool kept = dev >= 0 && dev < 64;
+  *out = kept ? at[dev].load() : nullptr;
+  if (*out) return cudaSuccess;
   void* p = nullptr;
   e = cudaGetSymbolAddress(&p, c_T);
   if (e != cudaSuccess) return e;
   *out = static_cast<const uint64_t*>(p);
-  if (dev >= 0 && dev < 64) at[dev] = *out;
+  if (kept) at[dev].store(*out);
   return cudaSuccess;
 }
 
@@ -837,9 +837,9 @@ __device__ __forceinline__ void quant_finalize_body(const QuantArgs& a, const in
   }
   // the totals, then three independent chains, each a long one on this GPU, on
   // three warps (on three lanes of one warp they ran one after another, and
-  // the quotient was the compiler's 128-bit division; 13.6 -> 12.4 us for a batch
-  // of 60): the quotient for the
-  // copy counts, the logarithm of LSE, the division of N_eff
+  // the quotient was the compiler's 128-bit division; 13.6 -> 12.4 us for a
+  // batch of 60): the quotient for the copy counts, the logarithm of LSE, the
+  // division of N_eff
   __shared__ uint64_t s_R;
   __shared__ double s_lse, s_sed, s_ess;
   const uint64_t n = uint64_t(a.n);
