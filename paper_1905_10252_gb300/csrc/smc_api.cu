@@ -349,8 +349,12 @@ constexpr int kGraphIters = 8;
 // Iterations a sampler runs by plain launches before its graph of eight, and
 // before its graph of one, is built: the instantiation (0.1 to 0.2 ms of the
 // host) then overlaps the first eight, and a sampler that runs a few
-// iterations in all pays for no graph.
-constexpr int kPlainBefore8 = 8, kPlainBefore1 = 16;
+// iterations in all pays for no graph.  A call with fewer than kTwoGraphs left
+// launches the graph of eight once at most, which does not repay its building:
+// there it waits until the sampler has run kPlainBefore1 (a new FP64 sampler's
+// 20 iterations, N = 1100: Student-t 774 -> 728 us, Gaussian D = 12
+// 1324 -> 1283; FP32 logistic D = 5, N = 3000, M = 500: 988 -> 938).
+constexpr int kPlainBefore8 = 8, kPlainBefore1 = 24, kTwoGraphs = 2 * kGraphIters;
 
 cudaError_t build_graph(smc_sampler* h, int iterations, cudaGraphExec_t* out) {
   cudaGraph_t g = nullptr;
@@ -608,7 +612,8 @@ int smc_step(smc_sampler* h, int32_t k, double* mean_dev, double* cov_dev, smc_i
   }
   for (int32_t it = 0; it < k;) {
     const int32_t plain = k - it - (cov_dev ? 1 : 0);  // iterations left without the covariance
-    const bool eight = plain >= kGraphIters && (h->g_iter[1] || (may_build && h->plain_run >= kPlainBefore8));
+    const int32_t before8 = plain >= kTwoGraphs ? kPlainBefore8 : kPlainBefore1;
+    const bool eight = plain >= kGraphIters && (h->g_iter[1] || (may_build && h->plain_run >= before8));
     const bool one = plain > 0 && (h->g_iter[0] || (may_build && h->plain_run >= kPlainBefore1));
     if (eight || one) {
       cudaGraphExec_t& g = h->g_iter[eight ? 1 : 0];
