@@ -524,7 +524,18 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// Stores v at p's place in the shared memory of the cluster's block 0.
+// The same barrier in two halves, for the start: shared memory of another
+// block may only be accessed once that block runs.  Arriving on entry and
+// waiting just before the first such access leaves the work between them to
+// hide the wait.
+__device__ __forceinline__ void cluster_arrive_started() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait_started() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Stores v at p's place in the shared memory of the cluster's block 0, which
+// has started (cluster_wait_started).
 __device__ __forceinline__ void st_rank0(uint64_t* p, uint64_t v) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(uint32_t(__cvta_generic_to_shared(p))));
@@ -567,6 +578,7 @@ __device__ __forceinline__ void load_cols(const double* __restrict__ row, int c,
 
 template <typename ST, int CW, bool EST>
 __global__ void __launch_bounds__(kQThreads, 2) __cluster_dims__(kQSplit, 1, 1) k_quant_reduce_cluster(QuantArgs a) {
+  cluster_arrive_started();
   chain_begin();
   __shared__ QuantClusterSmem sm;
   const int s = int(cluster_rank());
@@ -642,6 +654,7 @@ __global__ void __launch_bounds__(kQThreads, 2) __cluster_dims__(kQSplit, 1, 1) 
     sm.sh[wid][4] = uint64_t(se >> 64);
   }
   __syncthreads();
+  cluster_wait_started();  // every block of the cluster runs: block 0 may be written
   if (tid == 0) {
     uint64_t tw = 0;
     u128 t2 = 0, te = 0;
