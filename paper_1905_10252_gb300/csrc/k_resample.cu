@@ -2093,7 +2093,7 @@ cudaError_t launch_max_logw(const double* logw, int64_t n, DevState* st, cudaStr
 // D = 8 17 -> 28 and scan 13.0 -> 15.5 us, 4096 tiles 0.129 -> 0.50 ms (several
 // waves of blocks that each wait for the weights, their cluster and shared
 // memory of another SM).
-bool quant_split(int64_t n) { return qblocks(n) <= kQSplitTiles; }
+static bool quant_split(int64_t n) { return qblocks(n) <= kQSplitTiles; }
 
 template <typename ST>
 static cudaError_t quant_reduce_t(const QuantArgs& a, cudaStream_t s) {

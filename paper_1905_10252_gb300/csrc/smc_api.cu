@@ -32,6 +32,11 @@ int quant_shift(int64_t n) {
   return F > 62 ? 62 : F;
 }
 
+// Words of QuantArgs::csub.  Larger samplers do not use it; they keep the room of
+// the largest that does, so that no workspace is smaller than one for fewer
+// particles (a caller may size it once, for its largest N).
+size_t csub_words(int64_t n) { return size_t(std::min<int64_t>(div_up(n, kQTile), kQSplitTiles)) * kQSplit; }
+
 // two_rs: a second run-start array (SMC_FLAG_DEFER_REDISTRIBUTE samplers)
 Layout layout_for(int64_t n, int d, int m = 0, bool two_rs = false) {
   Layout L{};
@@ -53,7 +58,7 @@ Layout layout_for(int64_t n, int d, int m = 0, bool two_rs = false) {
   L.cbase = p;
   p = align_up(p + size_t(L.qblocks) * sizeof(uint64_t));
   L.csub = p;
-  if (quant_split(n)) p = align_up(p + size_t(L.qblocks) * kQSplit * sizeof(uint64_t));
+  p = align_up(p + csub_words(n) * sizeof(uint64_t));
   L.xpart = p;
   p = align_up(p + size_t(L.qblocks) * size_t(d < 1 ? 1 : d) * sizeof(double));
   L.rs = p;
@@ -748,7 +753,7 @@ RawLayout raw_layout(int64_t n) {
   L.cbase = p;
   p = align_up(p + size_t(L.qblocks) * sizeof(uint64_t));
   L.csub = p;
-  if (quant_split(n)) p = align_up(p + size_t(L.qblocks) * kQSplit * sizeof(uint64_t));
+  p = align_up(p + csub_words(n) * sizeof(uint64_t));
   L.rs = p;
   p = align_up(p + size_t(n) * sizeof(int32_t));
   L.wbuf = p;

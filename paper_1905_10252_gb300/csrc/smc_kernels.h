@@ -252,7 +252,6 @@ cudaError_t launch_take_errors_batch(const ParticleArgs* pa, int32_t* errs, int 
 cudaError_t upload_expfx_table();  // once per device, outside stream capture
 cudaError_t expfx_table(const uint64_t** out);  // its device address (after the upload)
 cudaError_t launch_max_logw(const double* logw, int64_t n, DevState* st, cudaStream_t s);
-bool quant_split(int64_t n);  // csub is used at this size
 cudaError_t launch_quant_reduce(const QuantArgs& a, cudaStream_t s);
 cudaError_t launch_quant_finalize(const QuantArgs& a, int set_lse_prev, cudaStream_t s);
 cudaError_t launch_quant_scan(const QuantArgs& a, cudaStream_t s);
