@@ -198,11 +198,13 @@ __device__ __forceinline__ uint32_t img_off(int r, int k) {
   return uint32_t((r >> 3) * 512 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2);
 }
 
-// FP64 value of a finite FP32 number by its bits (no conversion instruction,
-// which would take a slot of the FP64 pipe); zero and subnormals aside.
+// FP64 value of an FP32 number by its bits (no conversion instruction, which
+// would take a slot of the FP64 pipe); zeros, subnormals, infinities and NaN
+// (exponent field 0 or 255) are converted.  (The GPU's own NaN, 0x7FFFFFFF,
+// rounds to -0 in the BF16 images: this is the way on which it reaches log pi.)
 __device__ __forceinline__ double widen(float f) {
   const uint32_t u = __float_as_uint(f);
-  if ((u & 0x7F800000u) == 0) return double(f);
+  if (((u + 0x00800000u) & 0x7F000000u) == 0) return double(f);
   return __hiloint2double(int((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), int(u << 29));
 }
 
