@@ -38,7 +38,7 @@
 // one try_wait, each warp has its next 16 columns on the way across half
 // tiles, and the loop holds no FP64 instruction (2 lanes per SM and clock;
 // the flush of the sums to FP64 took a sixth of the time): sums of up to 8
-// data tiles are added up as exact FP32 pairs (two-sum).
+// data tiles are added up as pairs of FP32 values (two-sum).
 // N = 2^18, M = 8192, D = 32: 0.500 -> 0.394 ms, 13.6 -> 18.4 elements per SM
 // and clock.
 //
@@ -208,13 +208,22 @@ __device__ __forceinline__ double widen(float f) {
   return __hiloint2double(int((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), int(u << 29));
 }
 
-// (hi, lo) += v without rounding (two-sum; lo takes the exact remainders).
-__device__ __forceinline__ void add_exact(float v, float& hi, float& lo) {
+// (hi, lo) += v: two-sum, so hi's rounding error is exact; only the additions
+// of those errors into lo round (2^-24 of 2^-24 of the sum).
+__device__ __forceinline__ void add_pair(float v, float& hi, float& lo) {
   const float s = __fadd_rn(hi, v);
   const float b = __fsub_rn(s, hi);
   lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(v, b)));
   hi = s;
 }
+// The FP64 value of such a sum.  An infinite hi stands alone: the two-sum's
+// error is then inf - inf.
+__device__ __forceinline__ double pair_value(float hi, float lo) {
+  return isinf(hi) ? double(hi) : double(hi) + double(lo);
+}
+// The sums of |z| are kept at this scale, so that a total of finite partial
+// sums (2^20 of them at most: M < 2^31) stays finite, as it did in FP64.
+constexpr float kAbsScale = 0x1p-24f;
 
 __global__ void __launch_bounds__(kTcThreads, 1) k_logistic_tc(ParticleArgs a) {
   chain_begin();
@@ -471,7 +480,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_logistic_tc(ParticleArgs a) {
         lw0 = a.logw[i];
         lp0 = lp[i];
       }
-      // sums over up to 8 image tiles, and their exact totals
+      // sums over up to 8 image tiles, and their totals as FP32 pairs
       float fabs4[2] = {0.0f, 0.0f}, flg4[2] = {0.0f, 0.0f};
       float sa[2] = {0.0f, 0.0f}, sal[2] = {0.0f, 0.0f}, sg[2] = {0.0f, 0.0f}, sgl[2] = {0.0f, 0.0f};
       // A warp always has the load of its next 32 columns in flight, across
@@ -522,8 +531,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_logistic_tc(ParticleArgs a) {
         if ((j & 7) == 7 || j == nx - 1) {
 #pragma unroll
           for (int p = 0; p < 2; ++p) {
-            add_exact(fabs4[p], sa[p], sal[p]);
-            add_exact(flg4[p], sg[p], sgl[p]);
+            add_pair(fabs4[p] * kAbsScale, sa[p], sal[p]);
+            add_pair(flg4[p], sg[p], sgl[p]);
             fabs4[p] = flg4[p] = 0.0f;
           }
         }
@@ -531,8 +540,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_logistic_tc(ParticleArgs a) {
       double acc_abs[2], acc_lg[2];
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
-        acc_abs[p] = double(sa[p]) + double(sal[p]);
-        acc_lg[p] = double(sg[p]) + double(sgl[p]);
+        acc_abs[p] = pair_value(sa[p], sal[p]) * (1.0 / double(kAbsScale));
+        acc_lg[p] = pair_value(sg[p], sgl[p]);
       }
       double* sp = s_part + (tl * kTcPT + row) * 4;
       if (hh == 1) {
