@@ -19,9 +19,12 @@
 // 4.2.2), 11 FP32 operations per pair, and the weight comes from the integer
 // exponential of the quantise pass with its exponent kept apart, so that a
 // weight far below the largest keeps its relative precision.  The sums
-// carry about 2^-45 relative error, far below the 2^-25 of rounding a row's
+// carry about 2^-45 relative error (with k rows per thread at most k^2 2^-48),
+// far below the 2^-25 of rounding a row's
 // difference to FP32 (the row precision), and no FP64 operation is left on
-// the per-pair path.  FP64 samplers use FP64 FMAs, one per pair.
+// the per-pair path.  FP64 samplers use FP64 FMAs, one per pair.  A block whose
+// values or weights leave the range in which that holds (needs_fp64) is summed
+// again in FP64.
 //
 // Measured (kernel alone): N = 2^20, D = 32 FP32 4.59 -> 0.33 ms (0.79 of the
 // issue slots, 0.64 of the FP32 pipe); N = 2000003, D = 12 1.67 -> 0.165 ms.
@@ -101,10 +104,70 @@ __device__ __forceinline__ float centred(float x, float mh, float ml) {
   return __fadd_rn(d, __fsub_rn(e, ml));
 }
 
+// The exponent of s (sums are kept at 2^-e of the weights e^{log w - m}, so that
+// they reach no further than with w~ itself).
+__device__ __forceinline__ int sum_exponent(double s) {
+  const int e = (__double2hiint(s) >> 20) - 1023;
+  return e > -1023 && e < 1024 ? e : 0;
+}
+
+// Whether a block's FP32 sums of a column may be off by more than 2^-36 of
+// them, from the scaled column's largest |value| (its bits) and its sum of
+// squares s.  Values stay below 2^40, so that no sum of 2^23 rows overflows.
+// Weights below 2^-120 of the largest count as zero (at most 2^23 2^-120
+// max^2), and additions below 2^-126 lose bits (2^23 2^-149 max).  Both are
+// small against s unless the heavy rows' values are far below the largest one.
+__device__ __forceinline__ bool needs_fp64(int max_bits, double s) {
+  if (max_bits == 0) return false;
+  const int R = (max_bits >> 23) - 126;  // max < 2^R
+  if (R > 40) return true;
+  const int least = max(2 * R - 61, max(R, 0) - 88);
+  return !(s >= scalbn(1.0, least) && s < INFINITY);
+}
+
+// A block's sums in FP64, one pair per thread and turn: products and sums of
+// FP64 values, the rows' differences rounded to FP32 as on the fast path.  FP64
+// units bound it; only the blocks that need it come here (all of them at
+// N = 2^20, D = 32: 4.7 ms beside the 0.33 of the fast path).
+__device__ __noinline__ void block_fp64(const ParticleArgs& a, const float* __restrict__ x, int rows, double scale,
+                                        float* s_r, double* s_w, double* __restrict__ out) {
+  const int d = a.d, npairs = d * (d + 1) / 2, tid = threadIdx.x;
+  const double m = a.st->m;
+  const double* const mean = a.st->mean;
+  constexpr int kPairs = (kMaxD * (kMaxD + 1) / 2 + kCovThreads - 1) / kCovThreads;
+  double acc[kPairs] = {};
+  int ca[kPairs], cb[kPairs];
+  for (int k = 0; k < kPairs; ++k) {
+    int p = min(tid + k * kCovThreads, npairs - 1);
+    ca[k] = 0;
+    while (p >= d - ca[k]) {
+      p -= d - ca[k];
+      ++ca[k];
+    }
+    cb[k] = ca[k] + p;
+  }
+  for (int64_t base = int64_t(blockIdx.x) * rows; base < a.n; base += int64_t(gridDim.x) * rows) {
+    const int have = int(a.n - base < rows ? a.n - base : int64_t(rows));
+    for (int e = tid; e < have * d; e += kCovThreads) s_r[e] = float(double(x[base * d + e]) - mean[e % d]);
+    if (tid < have) {
+      const double lw = a.logw[base + tid];
+      s_w[tid] = lw == -INFINITY ? 0.0 : exp(lw - m) * scale;
+    }
+    __syncthreads();
+    for (int k = 0; k < kPairs; ++k)
+      if (tid + k * kCovThreads < npairs)
+        for (int r = 0; r < have; ++r)
+          acc[k] = fma(s_w[r] * double(s_r[r * d + ca[k]]), double(s_r[r * d + cb[k]]), acc[k]);
+    __syncthreads();
+  }
+  for (int k = 0; k < kPairs; ++k)
+    if (tid + k * kCovThreads < npairs) out[tid + k * kCovThreads] = acc[k];
+}
+
 // Partial sums covpart[block][pair] (pairs a <= b row by row).  The FP32
 // path works on columns scaled by powers of two taken from the first rows
 // (every block the same) and, in each block, on weights scaled by a running
-// power of two, so that sums of any magnitude stay clear of FP32's limits.
+// power of two.
 template <typename T>
 __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const double* cov,
                                                       double* __restrict__ covpart,
@@ -125,11 +188,14 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
   __shared__ int s_ex[kMaxD];
   __shared__ uint64_t s_T[kF32 ? 128 : 1];
   __shared__ int s_emax[2];
+  __shared__ int s_max[kF32 ? kMaxD : 1];  // FP32: the columns' largest |value| (scaled; its bits)
+  __shared__ int s_redo;
   const int tid = threadIdx.x;
   const int d = a.d, nt = (d + kTileC - 1) / kTileC, nc = nt * kTileC;
   const int64_t n = a.n;
   const T* __restrict__ x = static_cast<const T*>(a.st->cur ? a.x[1] : a.x[0]);
   const double m = a.st->m;
+  const int se = sum_exponent(a.st->est_s);
   const int tiles = cov_tiles(nt), groups = kCovThreads / tiles;
   const int rows = min(S::kCap / nc, kCovThreads) / groups * groups;
   // a thread stages one column's values of rows er, er + sr, ... (the first
@@ -141,7 +207,9 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
     s_mh[tid] = T(mu);
     s_ml[tid] = T(mu - double(T(mu)));
     s_ex[tid] = 0;
+    if (kF32) s_max[tid] = 0;
   }
+  if (tid == 0) s_redo = 0;
   if (kF32 && tid < 128) s_T[tid] = exp_table[tid];
   if (tid < 2) s_emax[tid] = -(1 << 20);
   for (int k = tid; k < S::kCap; k += kCovThreads) {  // (columns d .. nc stay zero)
@@ -183,6 +251,8 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
     if (kF32) inv = s_inv[ec];
   }
   int K = -(1 << 20);  // FP32: weights are scaled by 2^-K
+  int vmax = 0;        // FP32: the largest |value| this thread staged (its bits)
+  const double scale = scalbn(1.0, -se);
   int turn = 0;
   // a chunk's values and log-weights are loaded while the one before it is
   // summed
@@ -230,7 +300,7 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
       const float f = K - E > 120 ? 0.0f : __int_as_float((127 - (K - E)) << 23);
       s_wf[tid] = make_float2(h * f, l * f);
     } else {
-      s_wd[tid] = lw == -INFINITY ? 0.0 : exp(lw - m);
+      s_wd[tid] = lw == -INFINITY ? 0.0 : exp(lw - m) * scale;
     }
     __syncthreads();
 #pragma unroll
@@ -242,6 +312,7 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
           const float2 w = s_wf[r];
           const float rv = r < have ? centred(v[q], mh, ml) * inv : 0.0f;
           const float u = __fmul_rn(w.x, rv);
+          vmax = max(vmax, __float_as_int(rv) & 0x7fffffff);
           s_r[at] = rv;
           s_u[at] = u;
           s_ul[at] = __fmaf_rn(w.y, rv, __fmaf_rn(w.x, rv, -u));
@@ -300,6 +371,8 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
   double* const red = reinterpret_cast<double*>(s_r);  // groups x tiles x 4 doubles
   static_assert(sizeof(s_r) >= size_t(kCovThreads) * kTileC * sizeof(double), "reduction space");
   const int npairs = d * (d + 1) / 2;
+  double* const out = covpart + size_t(blockIdx.x) * npairs;
+  if (kF32 && vmax) atomicMax(&s_max[ec], vmax);  // (seen behind the barriers below)
   int per = 32;
   while (per * tiles * kTileC > kCovThreads) per /= 2;
 #pragma unroll
@@ -321,12 +394,17 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov(ParticleArgs a, const do
       tile_of(k / kTileC, nt, ra, rb);
       const int ca = ra * kTileC + p, cb = rb * kTileC + k % kTileC;
       if (ca <= cb && cb < d) {
-        if (kF32) s = scalbn(s, K + s_ex[ca] + s_ex[cb]);
-        covpart[size_t(blockIdx.x) * npairs + ca * d - ca * (ca - 1) / 2 + (cb - ca)] = s;
+        if constexpr (kF32) {
+          if (ca == cb && needs_fp64(s_max[ca], K > -(1 << 20) ? s : 1.0)) s_redo = 1;
+          s = scalbn(s, K + s_ex[ca] + s_ex[cb] - se);
+        }
+        out[ca * d - ca * (ca - 1) / 2 + (cb - ca)] = s;
       }
     }
     __syncthreads();
   }
+  if constexpr (kF32)
+    if (s_redo) block_fp64(a, x, rows, scale, s_r, reinterpret_cast<double*>(s_wf), out);
 }
 
 // Sums the per-block partials, one warp per pair (lane l adds blocks l,
@@ -345,7 +423,7 @@ __global__ void __launch_bounds__(128) k_cov_finalize(const DevState* st, double
   for (int b = lane; b < nblocks; b += 32) v += covpart[size_t(b) * npairs + p];
   v = warp_sum(v);
   if (lane) return;
-  v /= st->est_s;
+  v /= scalbn(st->est_s, -sum_exponent(st->est_s));
   int ca = 0, k = p;
   while (k >= d - ca) {
     k -= d - ca;
