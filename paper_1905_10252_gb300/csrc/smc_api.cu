@@ -607,19 +607,19 @@ int smc_step(smc_sampler* h, int32_t k, double* mean_dev, double* cov_dev, smc_i
     }
     (void)cudaGetLastError();  // the grid cannot be resident here: separate launches below
   }
-  // (the legacy stream cannot be captured, nor one that the caller is capturing:
-  // there the iterations are plain launches unless their graph exists)
-  bool may_build = h->stream != nullptr;
-  if (may_build && !(h->g_iter[0] && h->g_iter[1])) {
+  // (the legacy stream cannot be captured; a stream that the caller is capturing
+  // takes neither a capture of ours nor the launch of a graph: plain launches)
+  bool graphs = h->stream != nullptr;
+  if (graphs) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     SMC_TRY(h, cudaStreamIsCapturing(h->stream, &cs));
-    may_build = cs == cudaStreamCaptureStatusNone;
+    graphs = cs == cudaStreamCaptureStatusNone;
   }
   for (int32_t it = 0; it < k;) {
     const int32_t plain = k - it - (cov_dev ? 1 : 0);  // iterations left without the covariance
     const int32_t before8 = plain >= kTwoGraphs ? kPlainBefore8 : kPlainBefore1;
-    const bool eight = plain >= kGraphIters && (h->g_iter[1] || (may_build && h->plain_run >= before8));
-    const bool one = plain > 0 && (h->g_iter[0] || (may_build && h->plain_run >= kPlainBefore1));
+    const bool eight = graphs && plain >= kGraphIters && (h->g_iter[1] || h->plain_run >= before8);
+    const bool one = graphs && plain > 0 && (h->g_iter[0] || h->plain_run >= kPlainBefore1);
     if (eight || one) {
       cudaGraphExec_t& g = h->g_iter[eight ? 1 : 0];
       if (!g) SMC_TRY(h, build_graph(h, eight ? kGraphIters : 1, &g));
