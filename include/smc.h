@@ -174,8 +174,8 @@ int smc_redistribute(smc_sampler* h, const int32_t* ncopies_dev);
  * with no host synchronisation between iterations (the decision stays on the
  * device; the launches are replayed from CUDA graphs once a sampler has run
  * its first iterations by plain launches).  An
- * FP64 sampler with N <= 256 (Gaussian or Student-t target) that does not
- * resample in every iteration runs the K
+ * FP64 sampler with D <= 2, N <= 512 or D = 3, N <= 256 (Gaussian or Student-t
+ * target) that does not resample in every iteration runs the K
  * iterations in one cooperative launch instead, with the same per-stage
  * arithmetic (bit-identical results); if its grid cannot be resident it uses
  * separate launches.

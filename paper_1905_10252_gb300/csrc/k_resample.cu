@@ -1814,16 +1814,16 @@ __global__ void __launch_bounds__(kRThreads) k_redistribute(RedistArgs a) {
 // ---------------------------------------------------------------- one-tile samplers
 // A fused small sampler that also returns the covariance
 // ends its last iteration with redistribute and commit as one kernel.
-template <typename V, int CPR>
+template <typename V>
 __global__ void __launch_bounds__(kRThreads) k_redistribute_commit(RedistArgs a, int d, int force_flip, int recycle) {
   __shared__ RedistSmemT<kRTile> sm;
-  redistribute_body<V, CPR, 8, false, kRTile>(a, 0, sm);
+  redistribute_body<V, 0, 8, false, kRTile>(a, 0, sm);
   __syncthreads();
   if (threadIdx.x < 32) commit_warp(a.st, d, force_flip, recycle);
 }
 
 // ---------------------------------------------------------------- fused small-sampler iterations
-// FP64 samplers of at most kSmallIter particles (see small_iter_fits): k
+// FP64 samplers of few particles and coordinates (see small_iter_fits): k
 // iterations of Algorithm 2 in one cooperative launch.  Every block runs its
 // share of the move + reweight with the particle-to-thread map of the
 // separate move launch (move_threads per block own particles); then block 0
@@ -1896,8 +1896,10 @@ union SmallIterSmem {
   RedistSmemT<kRTile> r;
 };
 
-template <int DMAX, typename V>
+template <typename V>
 __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
+  constexpr int DMAX = 4;  // (the separate kernels' width class)
+  static_assert(kSmallIterD <= DMAX, "coordinates");
   __shared__ SmallIterSmem sm;
   TargetSmem<double>& ts = sm.ts;
   QuantReduceSmem& qsm = sm.q;
@@ -1918,7 +1920,10 @@ __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
       __syncthreads();
       quant_finalize_body(s.q, 0);
       __syncthreads();
-      quant_scan_body<1>(s.q, 0, s.q.cbase[0], sm.sc);
+      if (s.a.n <= kQThreads)
+        quant_scan_body<1>(s.q, 0, s.q.cbase[0], sm.sc);
+      else
+        quant_scan_body<2>(s.q, 0, s.q.cbase[0], sm.sc);
       if (!(s.stop_last && it + 1 == s.k)) {
         __syncthreads();
         redistribute_body<V, 0, 8, true, kRTile>(s.r, 0, rsm);
@@ -1930,33 +1935,30 @@ __global__ void __launch_bounds__(kQThreads) k_iterate_small(SmallIterArgs s) {
   }
 }
 
-// Up to kSmallIter particles, unless every iteration resamples.  Measured per
-// iteration (fused, separate kernels): N = 64, D = 1 21.9, 24.3 us; N = 256, D = 1
-// 22.4, 23.9; N = 256, D = 4 29.2, 28.9; N = 1024, D = 4 32.0, 30.4; N = 2048, D = 32
-// 160, 111; and with a copy in every iteration N = 64, D = 1 26.7, 25.9, N = 256, D = 4
-// 32.2, 30.0 (block 0's stages one after another against many blocks each).
-static_assert(kSmallIter <= kRTile && kSmallIter <= kQThreads, "one copy tile, one scan item per thread");
-bool small_iter_fits(int64_t n, int dtype, int mode) {
-  return dtype == SMC_F64 && n <= kSmallIter && mode != SMC_RESAMPLE_ALWAYS;
-}
-
-template <int DMAX>
-static cudaError_t iterate_small_d(const SmallIterArgs& s, int blocks, cudaStream_t st) {
-  SmallIterArgs a = s;
-  void* args[] = {&a};
-  const void* fn = (s.r.row_bytes % 16 == 0) ? reinterpret_cast<const void*>(&k_iterate_small<DMAX, uint4>)
-                                             : reinterpret_cast<const void*>(&k_iterate_small<DMAX, uint2>);
-  return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(kQThreads), args, 0, st);
+// Few particles with few coordinates, unless every iteration resamples: block
+// 0 runs the stages one after another on its own, so it loses where they have
+// work to share out.  Measured per iteration (fused, separate kernels, us):
+//   D = 1  N = 64 21.8, 24.1   N = 256 22.4, 23.0   N = 512 24.1, 24.9
+//   D = 2  N = 64 20.0, 21.0   N = 256 21.5, 21.6   N = 300 22.5, 23.1   N = 512 22.8, 22.8
+//   D = 3  N = 64 23.1, 23.6   N = 256 25.4, 25.6   N = 300 26.1, 25.5
+//   D = 4  N = 64 24.1, 23.3   N = 256 26.2, 26.1   N = 512 28.3, 26.1
+//   D = 8  N = 64 36.6, 33.7   D = 32  N = 64 107.9, 102.0
+// and with a copy in every iteration D = 1  N = 64 25.1, 23.9, D = 3  N = 256 27.6, 27.5.
+static_assert(kSmallIter <= kRTile && kSmallIter <= 2 * kQThreads, "one copy tile, two scan items per thread");
+bool small_iter_fits(int64_t n, int d, int dtype, int mode) {
+  return dtype == SMC_F64 && mode != SMC_RESAMPLE_ALWAYS && n <= (d <= 2 ? kSmallIter : kSmallIter / 2) &&
+         d <= kSmallIterD;
 }
 
 cudaError_t launch_iterate_small(const SmallIterArgs& s, int move_blocks, cudaStream_t st) {
-  if (!small_iter_fits(s.a.n, s.a.dtype, s.q.mode) || s.k < 1 || move_blocks < 1 || s.move_threads < 1 ||
-      s.move_threads > kQThreads || s.d < 1 || s.d > kMaxD || s.r.row_bytes % 8 != 0)
+  if (!small_iter_fits(s.a.n, s.d, s.a.dtype, s.q.mode) || s.k < 1 || move_blocks < 1 || s.move_threads < 1 ||
+      s.move_threads > kQThreads || s.d < 1 || s.r.row_bytes % 8 != 0)
     return cudaErrorInvalidValue;
-  if (s.d <= 4) return iterate_small_d<4>(s, move_blocks, st);
-  if (s.d <= 8) return iterate_small_d<8>(s, move_blocks, st);
-  if (s.d <= 16) return iterate_small_d<16>(s, move_blocks, st);
-  return iterate_small_d<32>(s, move_blocks, st);
+  SmallIterArgs a = s;
+  void* args[] = {&a};
+  const void* fn = (s.r.row_bytes % 16 == 0) ? reinterpret_cast<const void*>(&k_iterate_small<uint4>)
+                                             : reinterpret_cast<const void*>(&k_iterate_small<uint2>);
+  return cudaLaunchCooperativeKernel(fn, dim3(move_blocks), dim3(kQThreads), args, 0, st);
 }
 
 // ---------------------------------------------------------------- batched launches
@@ -2208,20 +2210,11 @@ cudaError_t launch_redistribute(const RedistArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_redistribute_commit(const RedistArgs& a, int d, int force_flip, int recycle, cudaStream_t s) {
-  if (a.n > kRTile) return cudaErrorInvalidValue;
-  const int rb = a.row_bytes;
-  if (rb % 16 == 0) {
-    switch (rb / 16) {
-      case 1: k_redistribute_commit<uint4, 1><<<1, kRThreads, 0, s>>>(a, d, force_flip, recycle); break;
-      case 2: k_redistribute_commit<uint4, 2><<<1, kRThreads, 0, s>>>(a, d, force_flip, recycle); break;
-      case 4: k_redistribute_commit<uint4, 4><<<1, kRThreads, 0, s>>>(a, d, force_flip, recycle); break;
-      default: k_redistribute_commit<uint4, 0><<<1, kRThreads, 0, s>>>(a, d, force_flip, recycle); break;
-    }
-  } else if (rb % 8 == 0) {
-    k_redistribute_commit<uint2, 0><<<1, kRThreads, 0, s>>>(a, d, force_flip, recycle);
-  } else {
-    k_redistribute_commit<uint32_t, 0><<<1, kRThreads, 0, s>>>(a, d, force_flip, recycle);
-  }
+  if (a.n > kRTile || a.row_bytes % 8 != 0) return cudaErrorInvalidValue;
+  if (a.row_bytes % 16 == 0)
+    k_redistribute_commit<uint4><<<1, kRThreads, 0, s>>>(a, d, force_flip, recycle);
+  else
+    k_redistribute_commit<uint2><<<1, kRThreads, 0, s>>>(a, d, force_flip, recycle);
   return cudaGetLastError();
 }
 

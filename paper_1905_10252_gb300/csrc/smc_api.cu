@@ -512,7 +512,8 @@ int smc_init(smc_sampler** out, const smc_config* cfg, void* x_dev, void* x_alt_
   h->defer = (cfg->flags & SMC_FLAG_DEFER_REDISTRIBUTE) && est_in_move(h) && h->L.qblocks > 1;
   // small FP64 samplers (generic move kernel, one quantise block, one block's
   // copy): smc_step fuses their iterations into one cooperative launch
-  h->small_iter = small_iter_fits(h->n, h->dtype, cfg->resample_mode) && cfg->target != SMC_LOGISTIC && !h->defer;
+  h->small_iter =
+      small_iter_fits(h->n, h->d, h->dtype, cfg->resample_mode) && cfg->target != SMC_LOGISTIC && !h->defer;
   if (e != cudaSuccess) {
     int r = cuda_fail(nullptr, e, "smc_init launch");
     delete h;

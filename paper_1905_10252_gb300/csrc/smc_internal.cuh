@@ -31,7 +31,8 @@ constexpr int kQSplit = 8;            // blocks that share a tile in the passes 
 constexpr int kQSplitTiles = 76;       // ... of at most this many tiles
 constexpr int kRTile = 512;            // output rows per source entry (tile_src, stamps) of the redistribute copy
 constexpr int kCopyTile = 1024;        // output rows per block of the copy of large samplers and of batches
-constexpr int kSmallIter = 256;       // particles of a sampler whose iterations are one launch, at most
+constexpr int kSmallIter = 512;       // particles of a sampler whose iterations are one launch, at most,
+constexpr int kSmallIterD = 3;        // and its coordinates (small_iter_fits)
 constexpr int kRThreads = 256;
 constexpr int kPThreads = 256;        // particle kernels (init / move / reweight)
 constexpr int kFinThreads = 1024;     // single-block finalisers

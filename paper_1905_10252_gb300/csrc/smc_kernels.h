@@ -282,7 +282,7 @@ struct SmallIterArgs {
   int32_t stall;  // test hook (SMC_FLAG_TEST_STALL_BARRIER): the barrier waits for one block more than the grid
   int32_t pad;
 };
-bool small_iter_fits(int64_t n, int dtype, int mode);
+bool small_iter_fits(int64_t n, int d, int dtype, int mode);
 cudaError_t launch_iterate_small(const SmallIterArgs& s, int move_blocks, cudaStream_t st);
 int nearly_sort_tiles(int64_t n);
 cudaError_t launch_nearly_sort(const NearlySortArgs& a, cudaStream_t s);
