@@ -447,7 +447,7 @@ __device__ __forceinline__ void warp_write_est(float em, double R, float (&v)[DM
 // Algorithm 5 as a gather, for the 256 particles of move tile jt: row k of
 // the resampled set is row src(k) = the last run start at or before k
 // (rs[off_i] = i for every survivor i, -1 elsewhere).  tile_src holds src at
-// the first row of each kRTile output rows; run starts between that row and
+// the first of each 2^src_shift output rows; run starts between that row and
 // the move tile's first row are found by a backward search 32 rows at a time
 // (in all but heavily duplicated regions the 32 rows just before hold one).
 //
@@ -456,7 +456,7 @@ __device__ __forceinline__ void warp_write_est(float em, double R, float (&v)[DM
 // does not wait on memory:
 //   stage[0, 256)   rs[k0 .. k0 + 256)    (entries at or beyond n: masked)
 //   stage[256, 288) rs[k0 - 32 .. k0)     (the first step of the backward search)
-//   stage[288]      tile_src[k0 / kRTile]
+//   stage[288]      tile_src[k0 >> src_shift]
 // tile_sources_issue starts the copies; tile_sources_finish waits for them
 // and writes the tile's 256 sources to out[] (clamped into [0, n), as the copy
 // kernel clamps them).  Every lane of the warp takes part in both.
@@ -476,7 +476,8 @@ __device__ __forceinline__ void tile_sources_issue(const int32_t* __restrict__ r
                                                    int32_t* __restrict__ stage) {
   const int lane = threadIdx.x & 31;
   const int64_t k0 = jt * kEstTile;
-  const int64_t t0 = (k0 / kRTile) * kRTile;
+  const int sh = src_shift(n);
+  const int64_t t0 = (k0 >> sh) << sh;
   // lane l: entries [8l, 8l + 8) as two 16-byte pieces.  rs is 256-byte
   // aligned and padded to a multiple of 256 bytes, so a piece that starts
   // below n stays inside the array; pieces at or beyond n copy nothing
@@ -488,7 +489,7 @@ __device__ __forceinline__ void tile_sources_issue(const int32_t* __restrict__ r
     cp_async16(stage + 8 * lane + 4 * h, rs + (in ? k : 0), in ? 16 : 0);
   }
   if (k0 > t0) cp_async4(stage + kEstTile + lane, rs + (k0 - 32 + lane));
-  if (lane == 0) cp_async4(stage + kEstTile + 32, tile_src + k0 / kRTile);
+  if (lane == 0) cp_async4(stage + kEstTile + 32, tile_src + (k0 >> sh));
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
@@ -498,7 +499,8 @@ __device__ __forceinline__ void tile_sources_finish(const int32_t* __restrict__ 
   __syncwarp();  // every lane's copies have landed
   const int lane = threadIdx.x & 31;
   const int64_t k0 = jt * kEstTile;
-  const int64_t t0 = (k0 / kRTile) * kRTile;
+  const int sh = src_shift(n);
+  const int64_t t0 = (k0 >> sh) << sh;
   int carry = stage[kEstTile + 32];
   if (k0 > t0) {
     int m = stage[kEstTile + lane];

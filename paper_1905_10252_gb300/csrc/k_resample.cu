@@ -1194,20 +1194,22 @@ struct BigRuns {
 
 __device__ __forceinline__ void tile_starts_of_run(int32_t* __restrict__ tile_src, uint64_t lo, uint64_t hi,
                                                    uint64_t n, int32_t i, BigRuns& big) {
-  const uint64_t kb0 = ((lo + kRTile - 1) / kRTile) * kRTile;
+  const int sh = src_shift(int64_t(n));
+  const uint64_t rows = 1ull << sh;
+  const uint64_t kb0 = (lo + rows - 1) & ~(rows - 1);
   const uint64_t end = hi < n ? hi : n;
   if (kb0 >= end) return;
-  const uint64_t tiles = (end - kb0 + kRTile - 1) / kRTile;
+  const uint64_t tiles = (end - kb0 + rows - 1) >> sh;
   if (tiles > uint64_t(kBigRun)) {
     const int slot = atomicAdd(&big.count, 1);
     if (slot < kBigRuns) {
       big.src[slot] = i;
-      big.first[slot] = int64_t(kb0 / kRTile);
+      big.first[slot] = int64_t(kb0 >> sh);
       big.tiles[slot] = int64_t(tiles);
       return;
     }
   }
-  for (uint64_t kb = kb0; kb < end; kb += kRTile) tile_src[kb / kRTile] = i;  // (short run, or the queue is full)
+  for (uint64_t kb = kb0; kb < end; kb += rows) tile_src[kb >> sh] = i;  // (short run, or the queue is full)
 }
 
 __device__ __forceinline__ void tile_starts_flush(int32_t* __restrict__ tile_src, BigRuns& big) {
@@ -1462,9 +1464,9 @@ __global__ void __launch_bounds__(kQThreads) k_nc_reduce(NcScanArgs a) {
     a.part[blockIdx.x] = t | (bad ? kNcBad : 0);
   }
   // (stamped calls: this block's share of the stamps, zero until the scan)
-  constexpr int kStamps = kQTile / kRTile;
-  if (a.stamps && threadIdx.x < kStamps && blockIdx.x * kStamps + threadIdx.x < a.ntiles)
-    a.stamps[blockIdx.x * kStamps + threadIdx.x] = 0;
+  const int stamps = kQTile >> src_shift(a.n);
+  if (a.stamps && threadIdx.x < stamps && blockIdx.x * stamps + threadIdx.x < a.ntiles)
+    a.stamps[blockIdx.x * stamps + threadIdx.x] = 0;
 }
 
 __global__ void __launch_bounds__(kFinThreads) k_nc_finalize(NcScanArgs a) { chain_begin(); nc_finalize_body(a); }
@@ -1489,11 +1491,14 @@ constexpr uint64_t kFillAll = 1u << 17;
 __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
   chain_begin();
   if (a.st->err) return;
-  __shared__ int32_t win[kNcWin];
+  __shared__ __align__(16) int32_t win[kNcWin];
   __shared__ uint64_t scratch[33];
   __shared__ BigRuns big;
   __shared__ int s_nfill;
-  __shared__ int64_t s_fill[kFillTiles];
+  // (a window is staged or its tiles are queued, never both)
+  int64_t* const s_fill = reinterpret_cast<int64_t*>(win);
+  static_assert(sizeof(win) >= kFillTiles * sizeof(int64_t), "the queue's space");
+  const int sh = src_shift(a.n);
   __shared__ int s_has[kNcWin / kRTile + 2];  // staged window: its tiles that receive a run start
   if (threadIdx.x == 0) {
     big.count = 0;
@@ -1520,8 +1525,8 @@ __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
   if (staged) {
     for (int k = threadIdx.x; k < int(btot); k += blockDim.x) win[k] = -1;
   } else if (stamped && !fill_all && threadIdx.x == 0 && w0 < wend) {
-    s_fill[0] = int64_t(w0 / kRTile);  // the edge tiles, shared with the neighbouring windows
-    s_fill[1] = int64_t((wend - 1) / kRTile);
+    s_fill[0] = int64_t(w0 >> sh);  // the edge tiles, shared with the neighbouring windows
+    s_fill[1] = int64_t((wend - 1) >> sh);
     s_nfill = 2;
   }
   __syncthreads();
@@ -1531,8 +1536,8 @@ __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
       int64_t last = -1;
 #pragma unroll
       for (int q = 0; q < kQItems; ++q) {
-        if (c[q] > 0 && i0 + q < n && o < un && int64_t(o / kRTile) != last) {
-          last = int64_t(o / kRTile);
+        if (c[q] > 0 && i0 + q < n && o < un && int64_t(o >> sh) != last) {
+          last = int64_t(o >> sh);
           const int slot = atomicAdd(&s_nfill, 1);
           if (slot < kFillTiles) s_fill[slot] = last;
         }
@@ -1544,15 +1549,15 @@ __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
       for (uint64_t k = w0 + threadIdx.x; k < wend; k += blockDim.x) rsa[k] = -1;
     } else {
       for (int f = 0; f < s_nfill; ++f) {
-        const uint64_t t0 = max(w0, uint64_t(s_fill[f]) * kRTile);
-        const uint64_t t1 = min(wend, uint64_t(s_fill[f]) * kRTile + kRTile);
+        const uint64_t t0 = max(w0, uint64_t(s_fill[f]) << sh);
+        const uint64_t t1 = min(wend, (uint64_t(s_fill[f]) + 1) << sh);
         for (uint64_t k = t0 + threadIdx.x; k < t1; k += blockDim.x) rsa[k] = -1;
       }
     }
     __syncthreads();  // every -1 before any run start
     o = w0 + excl;
   }
-  const uint64_t tfirst = w0 / kRTile;
+  const uint64_t tfirst = w0 >> sh;
   int64_t stamped_tile = -1;  // (a thread's items are consecutive: one stamp per tile it reaches)
 #pragma unroll
   for (int q = 0; q < kQItems; ++q) {
@@ -1560,11 +1565,11 @@ __global__ void __launch_bounds__(kQThreads) k_nc_scan(NcScanArgs a) {
     if (c[q] > 0 && i < n && o < un) {
       if (staged) {
         win[o - w0] = int32_t(i);
-        if (stamped) s_has[o / kRTile - tfirst] = 1;
+        if (stamped) s_has[(o >> sh) - tfirst] = 1;
       } else {
         rsa[o] = int32_t(i);
-        if (stamped && int64_t(o / kRTile) != stamped_tile) {
-          stamped_tile = int64_t(o / kRTile);
+        if (stamped && int64_t(o >> sh) != stamped_tile) {
+          stamped_tile = int64_t(o >> sh);
           a.stamps[stamped_tile] = 1;
         }
       }
@@ -1690,7 +1695,7 @@ struct RedistSmemT {
 };
 using RedistSmem = RedistSmemT<kCopyTile>;
 
-// One tile of TILE output rows, a whole number of kRTile.
+// One tile of TILE output rows, which a source entry's rows divide.
 template <typename V, int CPR, int KU = 8, bool COH = false, int TILE = kCopyTile>
 __device__ __forceinline__ void redistribute_body(const RedistArgs& a, const int blk, RedistSmemT<TILE>& sm) {
   int cur = 0;
@@ -1710,19 +1715,20 @@ __device__ __forceinline__ void redistribute_body(const RedistArgs& a, const int
   int32_t* __restrict__ rs = rs_now(a.runstart, a.runstart_alt, a.st) + k0;
   constexpr int kItems = TILE / kRThreads;
   static_assert(TILE % kRTile == 0 && kRTile % kRThreads == 0, "whole rounds of the block per source entry");
+  const int sh = src_shift(n);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int32_t v[kItems];
 #pragma unroll
   for (int u = 0; u < kItems; ++u) {
     const int k = threadIdx.x + u * kRThreads;
-    // (a stamped stateless call: an unstamped kRTile has no run starts, and
-    // its slice is neither read nor reset)
-    const bool read = !a.stamps || (k < len && a.stamps[blk * (TILE / kRTile) + u * kRThreads / kRTile]);
+    // (a stamped stateless call: an unstamped entry's rows have no run starts,
+    // and their slice is neither read nor reset)
+    const bool read = !a.stamps || (k < len && a.stamps[(k0 + u * kRThreads) >> sh]);
     v[u] = (read && k < len) ? rs[k] : -1;
   }
   // the run covering the first output row may have started in an earlier tile
   const int32_t first =
-      threadIdx.x == 0 ? min(max(a.tile_src[int64_t(blk) * (TILE / kRTile)], 0), int32_t(n - 1)) : -1;
+      threadIdx.x == 0 ? min(max(a.tile_src[k0 >> sh], 0), int32_t(n - 1)) : -1;
 #pragma unroll
   for (int u = 0; u < kItems; ++u) {
     const int k = threadIdx.x + u * kRThreads;
@@ -2039,9 +2045,10 @@ __global__ void __launch_bounds__(kRThreads) k_identity_runs_batch(const RedistA
   const int64_t k0 = int64_t(m.y) * kCopyTile;
   const int len = int(a.n - k0 < kCopyTile ? a.n - k0 : int64_t(kCopyTile));
   int32_t* __restrict__ rs = rs_now(a.runstart, a.runstart_alt, a.st);
+  const int sh = src_shift(a.n);
   for (int k = threadIdx.x; k < len; k += kRThreads) {
     rs[k0 + k] = int32_t(k0 + k);
-    if (k % kRTile == 0) const_cast<int32_t*>(a.tile_src)[(k0 + k) / kRTile] = int32_t(k0 + k);
+    if ((k & ((1 << sh) - 1)) == 0) const_cast<int32_t*>(a.tile_src)[(k0 + k) >> sh] = int32_t(k0 + k);
   }
 }
 
@@ -2166,8 +2173,6 @@ cudaError_t launch_nc(const NcScanArgs& a, cudaStream_t s) {
   chain_launch(k_nc_scan, qblocks(a.n), kQThreads, 0, s, a);
   return cudaGetLastError();
 }
-
-constexpr int64_t kSmallCopy = 2 << 20;
 
 template <int TILE>
 static void redistribute_t(const RedistArgs& a, cudaStream_t s) {

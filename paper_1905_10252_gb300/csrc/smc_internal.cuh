@@ -29,8 +29,15 @@ constexpr int kQThreads = 256;        // 16 consecutive elements per thread
 constexpr int kQItems = kQTile / kQThreads;
 constexpr int kQSplit = 8;            // blocks that share a tile in the passes of small samplers
 constexpr int kQSplitTiles = 76;       // ... of at most this many tiles
-constexpr int kRTile = 512;            // output rows per source entry (tile_src, stamps) of the redistribute copy
-constexpr int kCopyTile = 1024;        // output rows per block of the copy of large samplers and of batches
+constexpr int kRTile = 512;            // output rows per block of the redistribute copy of up to kSmallCopy rows
+constexpr int kCopyTile = 1024;        // ... of larger ones and of batches
+constexpr int64_t kSmallCopy = 2 << 20;
+// log2 of the output rows per source entry (tile_src, stamps): the copy's own
+// tile.  (One entry per 512 rows at every size cost the scans of large samplers
+// the entries that no block reads: the copy-count passes at n = 2^24 took 90.5 us
+// with them, and their queue beside the window; 81.5 now.)
+__host__ __device__ constexpr int src_shift(int64_t n) { return n <= kSmallCopy ? 9 : 10; }
+static_assert(kRTile == 1 << src_shift(1) && kCopyTile == 1 << src_shift(kSmallCopy + 1), "an entry per copy tile");
 constexpr int kSmallIter = 512;       // particles of a sampler whose iterations are one launch, at most,
 constexpr int kSmallIterD = 3;        // and its coordinates (small_iter_fits)
 constexpr int kRThreads = 256;

@@ -183,7 +183,7 @@ struct NcScanArgs {
   int32_t clear_rs;     // the reduce pass sets runstart[0, n) to -1 first (runstart_alt NULL)
   int32_t reset_err;    // 1: the error word is this call's (set to its outcome); 0: an error is added to it
   // stamped calls (the stateless entry points above nc_small; zeroed by the
-  // reduce pass): per kRTile output rows, set when a run start lands in them -- runstart
+  // reduce pass): per 2^src_shift output rows, set when a run start lands in them -- runstart
   // then need not be clean on entry (k_nc_scan writes every slice the copy
   // reads); NULL: runstart must hold -1 everywhere on entry (above nc_small)
   int32_t* stamps;
