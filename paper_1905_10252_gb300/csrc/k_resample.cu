@@ -1975,6 +1975,11 @@ __device__ __forceinline__ int dclass(int d) { return d <= 4 ? 0 : (d <= 8 ? 1 :
 
 // left (standing batches of slots; NULL otherwise): see k_move_reweight_batch.
 // A slot's map covers its capacity; blocks past the member's own count exit.
+// WIDE: members of D > 16 too.  Their route has 32 column sums and as many loaded
+// values in registers (124 against 80 a thread), which costs the others a third
+// of their resident warps: two members of 2^22, D = 16 125 against 101 us, D = 4 100
+// against 85; six of 10^5, D = 32 31 with it, 42 before they had the route.
+template <bool WIDE>
 __global__ void __launch_bounds__(kQThreads) k_quant_reduce_batch(const QuantArgs* __restrict__ qa,
                                                                  const int4* __restrict__ map,
                                                                  const int32_t* __restrict__ left) {
@@ -1987,7 +1992,9 @@ __global__ void __launch_bounds__(kQThreads) k_quant_reduce_batch(const QuantArg
     case 0: quant_reduce_body<float, 4, true>(a, m.y, sm); break;
     case 1: quant_reduce_body<float, 8, true>(a, m.y, sm); break;
     case 2: quant_reduce_body<float, 16, true>(a, m.y, sm); break;
-    default: quant_reduce_body<float, 32, true>(a, m.y, sm); break;
+    default:
+      if constexpr (WIDE) quant_reduce_body<float, 32, true>(a, m.y, sm);
+      break;
   }
 }
 
@@ -2052,9 +2059,13 @@ __global__ void __launch_bounds__(kRThreads) k_identity_runs_batch(const RedistA
   }
 }
 
-cudaError_t launch_quant_reduce_batch(const QuantArgs* qa, const int4* map, int nblocks, cudaStream_t s,
+const void* quant_reduce_batch_kernel(bool wide) {
+  return wide ? reinterpret_cast<const void*>(&k_quant_reduce_batch<true>)
+              : reinterpret_cast<const void*>(&k_quant_reduce_batch<false>);
+}
+cudaError_t launch_quant_reduce_batch(const QuantArgs* qa, const int4* map, int nblocks, bool wide, cudaStream_t s,
                                       const int32_t* left) {
-  k_quant_reduce_batch<<<nblocks, kQThreads, 0, s>>>(qa, map, left);
+  (wide ? k_quant_reduce_batch<true> : k_quant_reduce_batch<false>)<<<nblocks, kQThreads, 0, s>>>(qa, map, left);
   return cudaGetLastError();
 }
 cudaError_t launch_quant_finalize_batch(const QuantArgs* qa, int count, cudaStream_t s, const int32_t* left) {

@@ -32,6 +32,7 @@ thread_local std::string g_batch_err = "ok";
 // Host-side block maps of a member list (independent of device addresses).
 struct Plan {
   int count = 0;
+  bool wide = false;                                    // a member has D > kNarrowD
   std::vector<int4> qmap;                               // quantise / scan blocks
   std::vector<int4> rmap;                               // copy tiles
   std::vector<int4> mmap[SMC_BATCH_MOVE_VARIANTS];      // move / reweight blocks, widest class first
@@ -52,6 +53,7 @@ Plan make_plan(smc_sampler* const* m, int count, int sms) {
   std::vector<double> w(count);
   double wsum = 0.0;
   for (int s = 0; s < count; ++s) {
+    p.wide = p.wide || m[s]->d > kNarrowD;
     order[s] = s;
     w[s] = double(m[s]->n) * double(m[s]->d + 8);  // ~ bytes and flops of the move per member
     wsum += w[s];
@@ -188,7 +190,7 @@ cudaError_t launch_batch_iteration(const smc_batch* b) {
     e = launch_move_reweight_classes(pa, b->at<GaussParamsF32>(b->L.gp), b->at<int4>(b->L.mmap[mv]),
                                      b->plan.mblocks[mv], s);
   if (e == cudaSuccess) e = launch_max_finalize_batch(pa, b->at<int32_t>(b->L.nb) + size_t(mv) * c, c, s);
-  if (e == cudaSuccess) e = launch_quant_reduce_batch(qa, qmap, nq, s);
+  if (e == cudaSuccess) e = launch_quant_reduce_batch(qa, qmap, nq, b->plan.wide, s);
   if (e == cudaSuccess) e = launch_quant_finalize_batch(qa, c, s);
   if (e == cudaSuccess) e = launch_quant_scan_batch(qa, qmap, nq, s);
   if (e == cudaSuccess)
@@ -395,7 +397,7 @@ int smc_batch_step_profile(smc_batch* b, void* const* events_host, int32_t n_eve
   BATCH_TRY(b, rec(1));
   BATCH_TRY(b, launch_max_finalize_batch(pa, b->at<int32_t>(b->L.nb) + size_t(mv) * c, c, s));
   BATCH_TRY(b, rec(2));
-  BATCH_TRY(b, launch_quant_reduce_batch(qa, qmap, nq, s));
+  BATCH_TRY(b, launch_quant_reduce_batch(qa, qmap, nq, b->plan.wide, s));
   BATCH_TRY(b, rec(3));
   BATCH_TRY(b, launch_quant_finalize_batch(qa, c, s));
   BATCH_TRY(b, rec(4));

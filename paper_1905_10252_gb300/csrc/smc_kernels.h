@@ -237,7 +237,11 @@ cudaError_t launch_max_finalize_batch(const ParticleArgs* pa, const int* nb, int
                                       const int32_t* left = nullptr);
 cudaError_t launch_begin_batch(const ParticleArgs* pa, int count, cudaStream_t s, const int32_t* left = nullptr);
 cudaError_t launch_commit_batch(const ParticleArgs* pa, int count, cudaStream_t s, int32_t* left = nullptr);
-cudaError_t launch_quant_reduce_batch(const QuantArgs* qa, const int4* map, int nblocks, cudaStream_t s,
+// wide: some member has more than kNarrowD coordinates (the kernel without it
+// does not reduce such a member)
+constexpr int kNarrowD = 16;
+const void* quant_reduce_batch_kernel(bool wide);
+cudaError_t launch_quant_reduce_batch(const QuantArgs* qa, const int4* map, int nblocks, bool wide, cudaStream_t s,
                                       const int32_t* left = nullptr);
 cudaError_t launch_quant_finalize_batch(const QuantArgs* qa, int count, cudaStream_t s, const int32_t* left = nullptr);
 cudaError_t launch_quant_scan_batch(const QuantArgs* qa, const int4* map, int nblocks, cudaStream_t s,

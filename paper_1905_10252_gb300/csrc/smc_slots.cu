@@ -230,7 +230,7 @@ cudaError_t launch_slots_iteration(const smc_slots* b) {
     e = launch_move_reweight_batch(pa, b->at<GaussParamsF32>(b->L.gp), b->at<int4>(b->L.mmap),
                                    int(b->plan.mmap.size()), s, left);
   if (e == cudaSuccess) e = launch_max_finalize_batch(pa, b->at<int32_t>(b->L.nb), c, s, left);
-  if (e == cudaSuccess) e = launch_quant_reduce_batch(qa, qmap, nq, s, left);
+  if (e == cudaSuccess) e = launch_quant_reduce_batch(qa, qmap, nq, true, s, left);
   if (e == cudaSuccess) e = launch_quant_finalize_batch(qa, c, s, left);
   if (e == cudaSuccess) e = launch_quant_scan_batch(qa, qmap, nq, s, left);
   if (e == cudaSuccess)
@@ -279,7 +279,8 @@ cudaError_t build_slots_graph(smc_slots* b) {
 
 // Compact maps of the attached slots (their own quantise / copy blocks and
 // the slot's move blocks), uploaded on the slots' stream, and the grid sizes
-// of the map-driven kernel nodes set to the new entry counts.
+// of the map-driven kernel nodes set to the new entry counts (and the
+// quantise reduce to the instance for the attached widths).
 cudaError_t write_compact_maps(smc_slots* b) {
   const size_t fq = b->plan.qmap.size(), fr = b->plan.rmap.size(), fm = b->plan.mmap.size();
   const int sb = b->stage_next;
@@ -290,6 +291,7 @@ cudaError_t write_compact_maps(smc_slots* b) {
   int4* r = q + fq;
   int4* m = r + fr;
   size_t nq = 0, nr = 0, nm = 0;
+  bool wide = false;
   // the creation order (largest capacity first), attached slots only
   std::vector<int> order(b->count);
   for (int s = 0; s < b->count; ++s) order[s] = s;
@@ -297,6 +299,7 @@ cudaError_t write_compact_maps(smc_slots* b) {
   for (int s : order) {
     const smc_sampler* h = b->m[s];
     if (!h) continue;
+    wide = wide || h->d > kNarrowD;
     const int hq = h->L.qblocks, hr = int(div_up(h->n, kCopyTile)), hm = b->plan.nb[s];
     for (int j = 0; j < hq; ++j) q[nq++] = make_int4(s, j, hq, 0);
     for (int j = 0; j < hr; ++j) r[nr++] = make_int4(s, j, hr, 0);
@@ -316,6 +319,7 @@ cudaError_t write_compact_maps(smc_slots* b) {
     e = cudaGraphKernelNodeGetParams(b->map_node[k], &kp);
     if (e != cudaSuccess) break;
     kp.gridDim = dim3(unsigned(counts[k]), 1, 1);
+    if (k == 1) kp.func = const_cast<void*>(quant_reduce_batch_kernel(wide));
     e = cudaGraphExecKernelNodeSetParams(b->graph, b->map_node[k], &kp);
   }
   if (e == cudaSuccess) b->dirty = false;
