@@ -353,7 +353,7 @@ int smc_batch_create(smc_batch** out, smc_sampler* const* members, int32_t count
  * HOST arrays of count DEVICE pointers (entries may be NULL) with the meaning
  * smc_step gives its arguments of those names, per member.  Iterations are
  * replayed from a CUDA graph of one batched iteration (one launch per stage,
- * the move one per width class). */
+ * the move one more for members of D = 8). */
 int smc_batch_step(smc_batch* b, int32_t k, double* const* mean_dev, smc_iter_stats* const* trace_dev,
                    double* const* fhat_dev);
 

@@ -807,6 +807,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_move_reweight_batch(const Part
                                                                      const GaussParamsF32* __restrict__ gps,
                                                                      const int4* __restrict__ map,
                                                                      const int32_t* __restrict__ left) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (see k_move_reweight_batch8)
   const int4 m = map[blockIdx.x];
   if (left && left[m.x] <= 0) return;
   const ParticleArgs a = pa[m.x];
@@ -825,18 +826,15 @@ __global__ void __launch_bounds__(kPThreads, 2) k_move_reweight_batch(const Part
     move_reweight_body<32, true, true, FactorSmem, false>(a, fs, m.y, m.z);
 }
 
-// The same for a batch whose map is sorted by width class: one launch per
-// class (up to 8, 16, 32 coordinates, and exactly as many), each with its own
-// registers.  In one kernel for all classes the widest class's
-// registers left no room for the D-exact ones (they spilled).  The launches
-// after the first start while it runs (their inputs are complete when the
-// first starts) and end after it: their last act is to wait for the launch
-// before them, so that whatever follows the last follows all.
-template <int DPL, bool FULL>
-__global__ void __launch_bounds__(kPThreads, 2) k_move_reweight_class(const ParticleArgs* __restrict__ pa,
-                                                                     const GaussParamsF32* __restrict__ gps,
-                                                                     const int4* __restrict__ map) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+// The same for a batch's members of D = 8: a D-exact kernel of its own (two
+// members of 2^22: 154 us against 169 in the kernel above; exact kernels for D =
+// 16 and 32 spill and were slower, 319 against 301 and 229 against 220 at 2^22 and
+// 2^20).  It starts while the other members' launch before it runs (their
+// inputs are complete when that one starts) and ends after it: its last act is
+// to wait for that launch, so that whatever follows this one follows both.
+__global__ void __launch_bounds__(kPThreads, 2) k_move_reweight_batch8(const ParticleArgs* __restrict__ pa,
+                                                                      const GaussParamsF32* __restrict__ gps,
+                                                                      const int4* __restrict__ map) {
   const int4 m = map[blockIdx.x];
   const ParticleArgs a = pa[m.x];
   __shared__ float4 sfac[kPairedFactor / 2];
@@ -844,7 +842,7 @@ __global__ void __launch_bounds__(kPThreads, 2) k_move_reweight_class(const Part
   stage_pairs(gps[m.x].P2, gps[m.x].mu, a.d, reinterpret_cast<float2*>(sfac), smu);
   __syncthreads();
   const FactorSmem fs{sfac, smu};
-  move_reweight_body<DPL, true, true, FactorSmem, DPL <= 16, false, FULL>(a, fs, m.y, m.z);
+  move_reweight_body<8, true, true, FactorSmem, true, false, true>(a, fs, m.y, m.z);
   if (blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -1042,27 +1040,14 @@ cudaError_t launch_move_reweight_batch(const ParticleArgs* pa, const GaussParams
 }
 cudaError_t launch_move_reweight_classes(const ParticleArgs* pa, const GaussParamsF32* gps, const int4* map,
                                          const int (&blocks)[kMoveClasses], cudaStream_t s) {
-  // (the first launch follows what is before it completely)
-  bool first = true;
   cudaError_t e = cudaSuccess;
-  auto one = [&](auto kernel, int n) {
-    if (n == 0 || e != cudaSuccess) return;
-    if (first) {
-      kernel<<<n, kPThreads, 0, s>>>(pa, gps, map);
-      e = cudaGetLastError();
-    } else {
-      e = chain_launch(kernel, n, kPThreads, 0, s, pa, gps, map);
-    }
-    first = false;
-    map += n;
-  };
-  one(k_move_reweight_class<32, true>, blocks[0]);
-  one(k_move_reweight_class<32, false>, blocks[1]);
-  one(k_move_reweight_class<16, true>, blocks[2]);
-  one(k_move_reweight_class<16, false>, blocks[3]);
-  one(k_move_reweight_class<8, true>, blocks[4]);
-  one(k_move_reweight_class<8, false>, blocks[5]);
-  return e;
+  if (blocks[0]) e = launch_move_reweight_batch(pa, gps, map, blocks[0], s);
+  if (e != cudaSuccess || blocks[1] == 0) return e;
+  map += blocks[0];
+  if (blocks[0]) return chain_launch(k_move_reweight_batch8, blocks[1], kPThreads, 0, s, pa, gps, map);
+  // (alone: after all that is before it)
+  k_move_reweight_batch8<<<blocks[1], kPThreads, 0, s>>>(pa, gps, map);
+  return cudaGetLastError();
 }
 cudaError_t launch_max_finalize_batch(const ParticleArgs* pa, const int* nb, int count, cudaStream_t s,
                                       const int32_t* left) {

@@ -35,8 +35,8 @@ struct Plan {
   bool wide = false;                                    // a member has D > kNarrowD
   std::vector<int4> qmap;                               // quantise / scan blocks
   std::vector<int4> rmap;                               // copy tiles
-  std::vector<int4> mmap[SMC_BATCH_MOVE_VARIANTS];      // move / reweight blocks, widest class first
-  int mblocks[SMC_BATCH_MOVE_VARIANTS][kMoveClasses] = {};  // of them per width class
+  std::vector<int4> mmap[SMC_BATCH_MOVE_VARIANTS];      // move / reweight blocks, by move_class
+  int mblocks[SMC_BATCH_MOVE_VARIANTS][kMoveClasses] = {};  // of them per class
   std::vector<int32_t> nb[SMC_BATCH_MOVE_VARIANTS];     // move blocks per member
 };
 
@@ -177,7 +177,7 @@ int bfail(smc_batch* b, int code, const std::string& msg) {
   } while (0)
 
 // One iteration of Algorithm 2 (lines 3-10) for every member: one launch per
-// stage, the move one per width class.
+// stage, the members of D = 8 a move of their own.
 cudaError_t launch_batch_iteration(const smc_batch* b) {
   const int c = b->count, mv = b->move_v;
   cudaStream_t s = b->stream;

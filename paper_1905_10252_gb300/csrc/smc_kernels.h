@@ -228,9 +228,10 @@ cudaError_t launch_logistic_tc(const ParticleArgs& a, int grid, cudaStream_t s);
 // decrements it.  NULL for plain batches (every member runs).
 cudaError_t launch_move_reweight_batch(const ParticleArgs* pa, const GaussParamsF32* gps, const int4* map, int nblocks,
                                        cudaStream_t s, const int32_t* left = nullptr);
-// a batch's map sorted by width class (move_class), blocks[c] of class c
-constexpr int kMoveClasses = 6;
-inline int move_class(int d) { return d > 16 ? (d == 32 ? 0 : 1) : (d > 8 ? (d == 16 ? 2 : 3) : (d == 8 ? 4 : 5)); }
+// a batch's map sorted by move_class, blocks[c] of class c (members of D = 8 last:
+// they have a kernel of their own)
+constexpr int kMoveClasses = 2;
+inline int move_class(int d) { return d == 8 ? 1 : 0; }
 cudaError_t launch_move_reweight_classes(const ParticleArgs* pa, const GaussParamsF32* gps, const int4* map,
                                          const int (&blocks)[kMoveClasses], cudaStream_t s);
 cudaError_t launch_max_finalize_batch(const ParticleArgs* pa, const int* nb, int count, cudaStream_t s,
