@@ -785,9 +785,9 @@ def run_batch(args):
             "stage_roofline": {"move_reweight": roof("move_reweight", mv_bytes),
                                "quantise_reduce_estimate": roof("quantise_reduce_estimate", q_bytes)},
             "stages_ms": {k: round(v, 5) for k, v in stage_ms.items()},
-            # begin, one move launch per width class, max, quantise reduce /
-            # finalise, scan, copy, commit
-            "gpu_launches": (7 + len({(d > 16) + (d > 8) + 3 * (d in (8, 16, 32)) for _, d in shapes})) * K,
+            # begin, move (members of D = 8 in a launch of their own), max,
+            # quantise reduce / finalise, scan, copy, commit
+            "gpu_launches": (7 + len({d == 8 for _, d in shapes})) * K,
             "clocks": clocks.summary(t_host0, t_host1),
         }
         print(json.dumps(line), flush=True)

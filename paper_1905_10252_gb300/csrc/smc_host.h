@@ -54,8 +54,8 @@ struct smc_sampler {
   bool gp_ready;
   // SMC_FLAG_DEFER_REDISTRIBUTE honoured: resampled rows are gathered by the next move
   bool defer;
-  // FP64 sampler of one quantise block and one copy tile: smc_step runs its
-  // iterations in one cooperative launch (k_iterate_small)
+  // small FP64 sampler (small_iter_fits): smc_step runs its iterations in one
+  // cooperative launch (k_iterate_small)
   bool small_iter;
   // CUDA graphs of one and of several iterations (without the covariance
   // stage), and the iterations run by plain launches so far (smc_step)
