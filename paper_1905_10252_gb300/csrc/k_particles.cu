@@ -46,13 +46,11 @@ __global__ void __launch_bounds__(32 * kSetupWarps) k_target_setup(TargetDev* tg
   constexpr int kW = kSetupWarps, kJ = DMAX / kW;
   __shared__ double sL[2 * DMAX][DMAX + 1];  // (rows DMAX .. are read past the last column: zero)
   __shared__ double sp[32];
-  __shared__ int s_bad;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     tg->kind = kind;
     tg->d = d;
     tg->nu = nu;
-    s_bad = 0;
   }
   if (threadIdx.x < d) {
     tg->mu[lane] = mu[lane];
@@ -75,16 +73,16 @@ __global__ void __launch_bounds__(32 * kSetupWarps) k_target_setup(TargetDev* tg
     for (int o = 0; o < kW; ++o) {
       const int k = base + o;
       if (k < d) {
+        bool bad = false;
         if (w == o) {
           const double v = __dsub_rn(row[0], acc[0]);
           double diag = 0.0;
           if (lane == k) diag = v > 0.0 ? __dsqrt_rn(v) : -1.0;
           diag = __shfl_sync(0xffffffffu, diag, k);
-          if (!(diag > 0.0)) s_bad = 1;  // not positive definite
+          bad = !(diag > 0.0);  // not positive definite
           if (lane < DMAX) sL[lane][k] = lane == k ? diag : (lane > k ? __ddiv_rn(v, diag) : 0.0);
         }
-        __syncthreads();
-        if (s_bad) {
+        if (__syncthreads_or(bad)) {  // (every warp leaves at the same column)
           if (threadIdx.x == 0) record_error(st, SMC_EINVAL);
           return;
         }
